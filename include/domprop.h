@@ -415,8 +415,10 @@ int64_t dp_debug_live_allocs(void);
  * lb_out, ub_out (which also hold the round state).  infeasible and rounds
  * are HOST pointers; params as for dp_propagate (NULL = defaults).  Work is
  * issued on `cuda_stream` (NULL = the legacy default stream); the host waits
- * for the stream after every round (one thread per row, no screen), so this
- * path is for callers that cannot allocate, not the fast path.
+ * for the stream after every round and the rounds have no screen and no
+ * marking, so this path is for callers that cannot allocate, not the fast
+ * path.  Rows of up to 256 nonzeros are summed in CSR order, longer ones by a
+ * block's threads in a fixed order of their own.
  *
  * Its only scratch -- the next-state bound keys and a control block -- is a
  * file-scope device array sized for n <= DP_NOALLOC_MAX_VARS variables

@@ -107,79 +107,297 @@ __global__ void k_na_prologue(int32_t m, int32_t n, const int64_t *row_ptr,
   }
 }
 
-// One round, one thread per row: the activity chain in CSR order, Step 2,
-// every nonzero's candidates (Eq. 3a/3b in residual form, Eq. 5a/5b, the
-// exactly-one-infinity rule), integer rounding and filtered atomics into the
-// next-state keys.  State is read from lo/hi (start of the round).
-__global__ void k_na_round(int32_t m, const int64_t *row_ptr, const int32_t *col,
-                           const double *val, const double *lhs_in, const double *rhs_in,
-                           const uint8_t *vt, const double *lo, const double *hi,
-                           long long *keys, NoallocCtrl *ctrl, double eps_int, double tau,
-                           double eps_feas, double thr) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= m) return;
-  const double lhs = side_norm(lhs_in[i], thr), rhs = side_norm(rhs_in[i], thr);
-  const int64_t b = row_ptr[i], e = row_ptr[i + 1];
-  double minfin = 0.0, maxfin = 0.0;
-  int mininf = 0, maxinf = 0;
-  for (int64_t k = b; k < e; ++k) {
-    const double a = val[k];
-    const int32_t j = col[k];
-    const double bmin = a > 0.0 ? lo[j] : hi[j];
-    const double bmax = a > 0.0 ? hi[j] : lo[j];
-    if (is_inf_d(bmin)) ++mininf; else minfin = fma(a, bmin, minfin);
-    if (is_inf_d(bmax)) ++maxinf; else maxfin = fma(a, bmax, maxfin);
+// A row's sums and sides.
+struct NaRow {
+  double minfin, maxfin, lhs, rhs;
+  int mininf, maxinf;
+};
+
+struct NaArgs {
+  const int32_t *col;
+  const double *val;
+  const uint8_t *vt;
+  const double *lo, *hi;
+  long long *keys;
+  NoallocCtrl *ctrl;
+  double eps_int, tau, eps_feas, thr;
+};
+
+// One nonzero's contribution to the infinity counts; bn, bx: the bounds of
+// the finite sums (0 in the place of an infinite one).
+__device__ __forceinline__ void na_count(double a, double L, double U, NaRow &r, double &bn,
+                                         double &bx) {
+  const bool pos = __double2hiint(a) >= 0;
+  bn = pos ? L : U;
+  bx = pos ? U : L;
+  if (is_inf_d(bn)) {
+    ++r.mininf;
+    bn = 0.0;
   }
-  if (mininf == 0 && is_finite_d(rhs) && minfin > rhs + eps_feas * fmax(1.0, fabs(rhs)))
-    atomicExch(&ctrl->infeasible, 1);
-  if (maxinf == 0 && is_finite_d(lhs) && maxfin < lhs - eps_feas * fmax(1.0, fabs(lhs)))
-    atomicExch(&ctrl->infeasible, 1);
-  for (int64_t k = b; k < e; ++k) {
-    const double a = val[k];
-    const int32_t j = col[k];
-    const double L = lo[j], U = hi[j];
-    const double bmin = a > 0.0 ? L : U;
-    const double bmax = a > 0.0 ? U : L;
-    double resmin, resmax;
-    if (mininf == 0) resmin = fma(-a, bmin, minfin);
-    else if (mininf == 1 && is_inf_d(bmin)) resmin = minfin;
-    else resmin = -__longlong_as_double(0x7FF0000000000000ll);
-    if (maxinf == 0) resmax = fma(-a, bmax, maxfin);
-    else if (maxinf == 1 && is_inf_d(bmax)) resmax = maxfin;
-    else resmax = __longlong_as_double(0x7FF0000000000000ll);
-    bool hl = false, hu = false;
-    double lc = 0.0, uc = 0.0;
-    if (is_finite_d(rhs) && is_finite_d(resmin)) {
-      double c = (rhs - resmin) / a;
-      if (a > 0.0) { uc = c; hu = true; } else { lc = c; hl = true; }
+  if (is_inf_d(bx)) {
+    ++r.maxinf;
+    bx = 0.0;
+  }
+}
+
+// Step 2 of a row.
+__device__ __forceinline__ void na_step2(const NaArgs &A, const NaRow &r) {
+  if (r.mininf == 0 && is_finite_d(r.rhs) &&
+      r.minfin > r.rhs + A.eps_feas * fmax(1.0, fabs(r.rhs)))
+    atomicExch(&A.ctrl->infeasible, 1);
+  if (r.maxinf == 0 && is_finite_d(r.lhs) &&
+      r.maxfin < r.lhs - A.eps_feas * fmax(1.0, fabs(r.lhs)))
+    atomicExch(&A.ctrl->infeasible, 1);
+}
+
+// One nonzero's candidates (Eq. 3a/3b in residual form, Eq. 5a/5b, the
+// exactly-one-infinity rule), integer rounding and filtered atomics into the
+// next-state keys.
+__device__ __forceinline__ void na_candidates(const NaArgs &A, const NaRow &r, double a,
+                                              int32_t j, double L, double U) {
+  const bool pos = __double2hiint(a) >= 0;
+  const double bmin = pos ? L : U, bmax = pos ? U : L;
+  const bool have_r = is_finite_d(r.rhs) &&
+                      (r.mininf == 0 || (r.mininf == 1 && is_inf_d(bmin)));
+  const bool have_l = is_finite_d(r.lhs) &&
+                      (r.maxinf == 0 || (r.maxinf == 1 && is_inf_d(bmax)));
+  if (!have_r && !have_l) return;
+  bool hl = false, hu = false;
+  double lc = 0.0, uc = 0.0;
+  if (have_r) {
+    const double res = r.mininf == 0 ? fma(-a, bmin, r.minfin) : r.minfin;
+    if (is_finite_d(res)) {
+      const double c = (r.rhs - res) / a;
+      if (pos) { uc = c; hu = true; } else { lc = c; hl = true; }
     }
-    if (is_finite_d(lhs) && is_finite_d(resmax)) {
-      double c = (lhs - resmax) / a;
-      if (a > 0.0) { lc = c; hl = true; } else { uc = c; hu = true; }
+  }
+  if (have_l) {
+    const double res = r.maxinf == 0 ? fma(-a, bmax, r.maxfin) : r.maxfin;
+    if (is_finite_d(res)) {
+      const double c = (r.lhs - res) / a;
+      if (pos) { lc = c; hl = true; } else { uc = c; hu = true; }
     }
-    const bool isint = vt[j] != 0;
-    if (hl) {
-      if (isint) lc = ceil(lc - eps_int);
-      if (!(fabs(lc) < thr)) hl = false;
+  }
+  const bool isint = A.vt[j] != 0;
+  if (hl) {
+    if (isint) lc = ceil(lc - A.eps_int);
+    if (!(fabs(lc) < A.thr)) hl = false;
+  }
+  if (hu) {
+    if (isint) uc = floor(uc + A.eps_int);
+    if (!(fabs(uc) < A.thr)) hu = false;
+  }
+  if (hl) {
+    const bool acc = is_inf_d(L) || (isint ? lc > L : lc > L + A.tau * fmax(1.0, fabs(L)));
+    if (acc) {
+      atomicMax(&A.keys[2 * (int64_t)j], okey(lc));
+      A.ctrl->changed = 1;
     }
-    if (hu) {
-      if (isint) uc = floor(uc + eps_int);
-      if (!(fabs(uc) < thr)) hu = false;
+  }
+  if (hu) {
+    const bool acc = is_inf_d(U) || (isint ? uc < U : uc < U - A.tau * fmax(1.0, fabs(U)));
+    if (acc) {
+      atomicMin(&A.keys[2 * (int64_t)j + 1], okey(uc));
+      A.ctrl->changed = 1;
     }
-    if (hl) {
-      bool acc = is_inf_d(L) || (isint ? lc > L : lc > L + tau * fmax(1.0, fabs(L)));
-      if (acc) {
-        atomicMax(&keys[2 * (int64_t)j], okey(lc));
-        ctrl->changed = 1;
+  }
+}
+
+constexpr int kNaThreads = 256;
+constexpr int kNaWarps = kNaThreads / 32;
+constexpr int kNaUnroll = 4;     // nonzeros whose loads are in flight together
+constexpr int kNaLaneRow = 32;   // longest row that one lane takes
+constexpr int kNaWarpRow = 256;  // longest row that one warp takes
+
+// Loads nonzeros k, k + step, ... (kNaUnroll of them, those below e).
+__device__ __forceinline__ void na_load(const NaArgs &A, int64_t k, int64_t step, int64_t e,
+                                        double (&a)[kNaUnroll], int32_t (&j)[kNaUnroll],
+                                        double (&L)[kNaUnroll], double (&U)[kNaUnroll]) {
+#pragma unroll
+  for (int u = 0; u < kNaUnroll; ++u) {
+    a[u] = 1.0;
+    j[u] = 0;
+    if (k + u * step < e) {
+      a[u] = A.val[k + u * step];
+      j[u] = A.col[k + u * step];
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < kNaUnroll; ++u) {
+    L[u] = U[u] = 0.0;
+    if (k + u * step < e) {
+      L[u] = A.lo[j[u]];
+      U[u] = A.hi[j[u]];
+    }
+  }
+}
+
+// A row by one lane: the activity chain in CSR order, Step 2, candidates.
+__device__ __forceinline__ void na_row_lane(const NaArgs &A, NaRow r, int64_t b, int64_t e) {
+  double a[kNaUnroll], L[kNaUnroll], U[kNaUnroll];
+  int32_t j[kNaUnroll];
+  for (int64_t k = b; k < e; k += kNaUnroll) {
+    na_load(A, k, 1, e, a, j, L, U);
+#pragma unroll
+    for (int u = 0; u < kNaUnroll; ++u)
+      if (k + u < e) {
+        double bn, bx;
+        na_count(a[u], L[u], U[u], r, bn, bx);
+        r.minfin = fma(a[u], bn, r.minfin);
+        r.maxfin = fma(a[u], bx, r.maxfin);
+      }
+  }
+  na_step2(A, r);
+  if (r.mininf > 1 && r.maxinf > 1) return;
+  for (int64_t k = b; k < e; k += kNaUnroll) {
+    na_load(A, k, 1, e, a, j, L, U);
+#pragma unroll
+    for (int u = 0; u < kNaUnroll; ++u)
+      if (k + u < e) na_candidates(A, r, a[u], j[u], L[u], U[u]);
+  }
+}
+
+// A row by one warp: 32 nonzeros are loaded side by side and added in CSR
+// order over shuffled values (lanes below 16 the minimum activity, the
+// others the maximum): the same chain as one lane's, bit for bit.
+__device__ __forceinline__ void na_row_warp(const NaArgs &A, NaRow r, int64_t b, int64_t e) {
+  const unsigned full = 0xFFFFFFFFu;
+  const int lane = threadIdx.x & 31;
+  double a[kNaUnroll], L[kNaUnroll], U[kNaUnroll];
+  int32_t j[kNaUnroll];
+  double fin = 0.0;
+  for (int64_t k = b; k < e; k += 32 * kNaUnroll) {
+    na_load(A, k + lane, 32, e, a, j, L, U);
+#pragma unroll
+    for (int u = 0; u < kNaUnroll; ++u) {
+      double bn = 0.0, bx = 0.0;
+      const int64_t k0 = k + 32 * u;
+      if (k0 + lane < e) na_count(a[u], L[u], U[u], r, bn, bx);
+      const int cnt = (int)(e - k0 < 32 ? e - k0 : 32);
+      for (int i = 0; i < cnt; ++i) {  // warp-uniform
+        const double av = __shfl_sync(full, a[u], i);
+        const double vn = __shfl_sync(full, bn, i), vx = __shfl_sync(full, bx, i);
+        fin = fma(av, lane < 16 ? vn : vx, fin);
       }
     }
-    if (hu) {
-      bool acc = is_inf_d(U) || (isint ? uc < U : uc < U - tau * fmax(1.0, fabs(U)));
-      if (acc) {
-        atomicMin(&keys[2 * (int64_t)j + 1], okey(uc));
-        ctrl->changed = 1;
+  }
+  r.minfin = __shfl_sync(full, fin, 0);
+  r.maxfin = __shfl_sync(full, fin, 16);
+  r.mininf = __reduce_add_sync(full, r.mininf);
+  r.maxinf = __reduce_add_sync(full, r.maxinf);
+  if (lane == 0) na_step2(A, r);
+  if (r.mininf > 1 && r.maxinf > 1) return;
+  for (int64_t k = b; k < e; k += 32 * kNaUnroll) {
+    na_load(A, k + lane, 32, e, a, j, L, U);
+#pragma unroll
+    for (int u = 0; u < kNaUnroll; ++u)
+      if (k + 32 * u + lane < e) na_candidates(A, r, a[u], j[u], L[u], U[u]);
+  }
+}
+
+// A row by the whole block: every thread adds its strided nonzeros in order,
+// then the threads' sums are added in a fixed tree, the same for every run.
+__device__ __forceinline__ void na_row_block(const NaArgs &A, NaRow r, int64_t b, int64_t e) {
+  __shared__ double s_min[kNaWarps], s_max[kNaWarps];
+  __shared__ int s_ni[kNaWarps], s_xi[kNaWarps];
+  const unsigned full = 0xFFFFFFFFu;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double a[kNaUnroll], L[kNaUnroll], U[kNaUnroll];
+  int32_t j[kNaUnroll];
+  for (int64_t k = b + threadIdx.x; k < e; k += kNaThreads * kNaUnroll) {
+    na_load(A, k, kNaThreads, e, a, j, L, U);
+#pragma unroll
+    for (int u = 0; u < kNaUnroll; ++u)
+      if (k + u * kNaThreads < e) {
+        double bn, bx;
+        na_count(a[u], L[u], U[u], r, bn, bx);
+        r.minfin = fma(a[u], bn, r.minfin);
+        r.maxfin = fma(a[u], bx, r.maxfin);
       }
-    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    r.minfin += __shfl_xor_sync(full, r.minfin, o);
+    r.maxfin += __shfl_xor_sync(full, r.maxfin, o);
+  }
+  r.mininf = __reduce_add_sync(full, r.mininf);
+  r.maxinf = __reduce_add_sync(full, r.maxinf);
+  if (lane == 0) {
+    s_min[warp] = r.minfin;
+    s_max[warp] = r.maxfin;
+    s_ni[warp] = r.mininf;
+    s_xi[warp] = r.maxinf;
+  }
+  __syncthreads();
+  r.minfin = s_min[0];
+  r.maxfin = s_max[0];
+  r.mininf = s_ni[0];
+  r.maxinf = s_xi[0];
+#pragma unroll
+  for (int w = 1; w < kNaWarps; ++w) {
+    r.minfin += s_min[w];
+    r.maxfin += s_max[w];
+    r.mininf += s_ni[w];
+    r.maxinf += s_xi[w];
+  }
+  __syncthreads();  // the sums are reused by the block's next row
+  if (threadIdx.x == 0) na_step2(A, r);
+  if (r.mininf > 1 && r.maxinf > 1) return;
+  for (int64_t k = b + threadIdx.x; k < e; k += kNaThreads * kNaUnroll) {
+    na_load(A, k, kNaThreads, e, a, j, L, U);
+#pragma unroll
+    for (int u = 0; u < kNaUnroll; ++u)
+      if (k + u * kNaThreads < e) na_candidates(A, r, a[u], j[u], L[u], U[u]);
+  }
+}
+
+// One round, kNaThreads rows per block: short rows by a lane each, longer
+// ones by a warp, the longest by the block.  What bounds a round is the
+// latency of its longest row: one lane's walk takes about 1 us per nonzero
+// (two dependent loads and the binary64 chain), so a row of 12,000 nonzeros
+// took 12 ms per round where the block takes about 30 us.  A row of up to
+// kNaWarpRow nonzeros is one FMA chain in CSR order whichever way it goes.
+__global__ void __launch_bounds__(kNaThreads)
+k_na_round(int32_t m, const int64_t *row_ptr, const double *lhs_in, const double *rhs_in,
+           NaArgs A) {
+  __shared__ int s_long[kNaThreads];
+  __shared__ int s_count;
+  if (threadIdx.x == 0) s_count = 0;
+  __syncthreads();
+  const int64_t i = blockIdx.x * (int64_t)kNaThreads + threadIdx.x;
+  NaRow r;
+  r.minfin = r.maxfin = r.lhs = r.rhs = 0.0;
+  r.mininf = r.maxinf = 0;
+  int64_t b = 0, e = 0;
+  if (i < m) {
+    r.lhs = side_norm(lhs_in[i], A.thr);
+    r.rhs = side_norm(rhs_in[i], A.thr);
+    b = row_ptr[i];
+    e = row_ptr[i + 1];
+    if (e - b <= kNaLaneRow) na_row_lane(A, r, b, e);
+    else if (e - b > kNaWarpRow) s_long[atomicAdd(&s_count, 1)] = threadIdx.x;
+  }
+  __syncwarp();
+  unsigned todo = __ballot_sync(0xFFFFFFFFu, e - b > kNaLaneRow && e - b <= kNaWarpRow);
+  for (; todo != 0u; todo &= todo - 1u) {
+    const int src = __ffs(todo) - 1;
+    NaRow q;
+    q.minfin = q.maxfin = 0.0;
+    q.mininf = q.maxinf = 0;
+    q.lhs = __shfl_sync(0xFFFFFFFFu, r.lhs, src);
+    q.rhs = __shfl_sync(0xFFFFFFFFu, r.rhs, src);
+    na_row_warp(A, q, __shfl_sync(0xFFFFFFFFu, b, src), __shfl_sync(0xFFFFFFFFu, e, src));
+  }
+  __syncthreads();
+  const int nlong = s_count;
+  for (int q = 0; q < nlong; ++q) {  // block-uniform
+    const int64_t row = blockIdx.x * (int64_t)kNaThreads + s_long[q];
+    NaRow x;
+    x.minfin = x.maxfin = 0.0;
+    x.mininf = x.maxinf = 0;
+    x.lhs = side_norm(lhs_in[row], A.thr);
+    x.rhs = side_norm(rhs_in[row], A.thr);
+    na_row_block(A, x, row_ptr[row], row_ptr[row + 1]);
   }
 }
 
@@ -308,15 +526,25 @@ extern "C" int dp_propagate_noalloc(int device, void *cuda_stream, int32_t m, in
     return DP_ERR_CUDA;
   if (h.err) return h.err;
 
+  NaArgs A{};
+  A.col = col_idx;
+  A.val = val;
+  A.vt = vartype;
+  A.lo = lb_out;
+  A.hi = ub_out;
+  A.keys = keys;
+  A.ctrl = ctrl;
+  A.eps_int = p.eps_int;
+  A.tau = p.tau_rel;
+  A.eps_feas = p.eps_feas;
+  A.thr = p.inf_threshold;
   int32_t r = 0;
   bool changed = false;
   for (; r < p.max_rounds;) {
     if (cudaMemsetAsync(ctrl, 0, sizeof(NoallocCtrl), st) != cudaSuccess) return DP_ERR_CUDA;
     if (m > 0)
-      k_na_round<<<(int)((m + 127) / 128), 128, 0, st>>>(m, row_ptr, col_idx, val, lhs, rhs,
-                                                          vartype, lb_out, ub_out, keys, ctrl,
-                                                          p.eps_int, p.tau_rel, p.eps_feas,
-                                                          p.inf_threshold);
+      k_na_round<<<(int)(((int64_t)m + kNaThreads - 1) / kNaThreads), kNaThreads, 0, st>>>(
+          m, row_ptr, lhs, rhs, A);
     if (n > 0)
       k_na_finish<<<(int)((n + 255) / 256), 256, 0, st>>>(n, vartype, keys, lb_out, ub_out, ctrl,
                                                           p.eps_feas);
