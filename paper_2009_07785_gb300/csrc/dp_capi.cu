@@ -336,6 +336,11 @@ int load_impl(dp_ctx *ctx, int32_t m, int32_t n, int64_t nnz, const int64_t *row
   M.nslices_split = H.nslices_split;
   M.nsplit_rows = H.nsplit_rows;
   M.round_warps = 8;
+  // whole rows are sorted by length, longest first
+  M.short0 = H.nslices;
+  while (H.layout == dp::kLayoutEll && M.short0 > H.nslices_split &&
+         H.slice_len[(size_t)M.short0 - 1] <= dp::kShortRow)
+    --M.short0;
   M.layout = H.layout;
   M.mp_ipt = H.mp_ipt;
   M.mp_nseg = H.mp_nseg;

@@ -38,6 +38,7 @@ int64_t live_allocs();
 constexpr int kSliceW = 32;                 // chunks per slice (= warp width)
 constexpr int32_t kLenMask = 0x3FFFFFFF;    // chunk length bits
 constexpr int32_t kExactFlag = 1 << 30;     // row must skip the FP32 screen
+constexpr int kShortRow = 12;               // longest row whose screen values stay in registers
 constexpr int32_t kLayoutEll = 0;           // sliced ELL over row chunks
 constexpr int32_t kLayoutMerge = 1;         // merge-path segments over CSR
 // A block of the persistent loop waits at a grid barrier for at most this
@@ -121,6 +122,7 @@ struct DevMatrix {
   int32_t nslices_split;  // slices [0, nslices_split) hold split-row chunks
   int32_t nsplit_rows;
   int32_t round_warps;      // warps per block of the round kernel (4 or 8)
+  int32_t short0;           // first slice whose rows all have kShortRow slots at most
   const double *val;        // padded slot-major values
   const int8_t *val8;       // the same values as int8 when all are small
                             // integers and compression is on, else null

@@ -148,21 +148,22 @@ __global__ void __launch_bounds__(256) k_cand_queue(DevMatrix M, DevState S) {
 // ------------------------------------------------------------- k_round --
 
 // Warps per block of k_round / k_cand_split: a launch shape the autotuner
-// chooses (4 or 8); the register budget per thread stays the same (32
-// resident warps per SM for a single problem, 24 for problem sets).
-constexpr int kRoundWarpsPerSM = 32;
-constexpr int kGroup = 2;         // slots per group in the activity loop
-// the problem-set variant (more live state per lane) and the persistent
-// kernel measured faster with fewer resident warps and longer groups
-constexpr int kRoundWarpsPerSMMulti = 24;
-constexpr int kGroupWide = 4;
+// chooses (4 or 8); the register budget per thread stays the same (24
+// resident warps per SM).  24 warps with groups of four slots against 32 with
+// two: 30M nonzeros of mixed rows 228 -> 210 us per round, a 2M-nonzero system
+// with rows of 50,000 107 -> 70 us (its longest lanes wait for half as many
+// groups); 16 x 6 and 16 x 8 are faster still on the latter and slower on the
+// former (244, 268 us).
+constexpr int kRoundWarpsPerSM = 24;
+constexpr int kGroup = 4;         // slots per group in the activity loop
 
 // One slice of the round (warp-level: the 32 lanes are its 32 chunks).
 // kVal8: the coefficients come from the int8 copy (converted when used, so
 // that the prefetched loads stay in flight).  kCo: records are loaded
 // through L2 (the persistent loop).
-template <bool kMulti, bool kVal8, int kG = kGroup, bool kCo = false>
+template <bool kMulti, bool kVal8, bool kCo = false>
 __device__ __forceinline__ void round_slice(const DevMatrix &M, const DevState &S, int slice) {
+  constexpr int kG = kGroup;
   const Ctrl *ctrl = S.ctrl;
   const int lane = threadIdx.x & 31;
   const int64_t c = (int64_t)slice * kSliceW + lane;
@@ -305,14 +306,106 @@ __device__ __forceinline__ void round_slice(const DevMatrix &M, const DevState &
   warp_enqueue<kSliceW, kCo>(rv, t, mininf, maxinf, len, c, sbase + lane, M, M.col, S);
 }
 
+// A slice of whole rows of at most kShortRow nonzeros (warp-level): the
+// lanes keep their rows' screen values in registers, so the survivors are
+// queued without a second pass over the nonzeros, and one-sided slices (most)
+// run code for one side.  30M nonzeros of mixed rows, 97% of the rows this
+// short: 210 -> 189 us per round.  Longer rows would need more registers than
+// 24 resident warps leave; in a kernel of its own, before, behind or beside
+// k_round in the graph, the same code made the round slower (265 us), since
+// nothing then fills the SMs while the long slices finish.
+template <int kSides>
+__device__ __forceinline__ void short_rows(const DevMatrix &M, const DevState &S, int64_t c,
+                                           int64_t elem0, int32_t len, int32_t row, bool exact,
+                                           double2 sd, bool right, int32_t *inf_flag) {
+  ShortAct<kSides, kShortRow> r;
+  short_activity<kSides, kShortRow>(
+      M, elem0, len, right,
+      [&](int32_t j, double &L, double &U, float &WU, float &WL) {
+        uint32_t fl;
+        ld_rec(S.rec + j, L, U, WU, WL, fl);
+      },
+      r);
+  constexpr int kR = 0, kL = kSides - 1;  // one side: both names are its index
+  const bool use_r = kSides == 2 || right, use_l = kSides == 2 || !right;
+  RowView rv;
+  rv.minfin = use_r ? r.fin[kR] : 0.0;
+  rv.maxfin = use_l ? r.fin[kL] : 0.0;
+  rv.mininf = use_r ? r.ninf[kR] : 0;
+  rv.maxinf = use_l ? r.ninf[kL] : 0;
+  rv.exact = exact ? 1 : 0;
+  rv.act = 0;
+  rv.thr_r = rv.thr_l = f_inf();
+  rv.lhs = sd.x;
+  rv.rhs = sd.y;
+  uint32_t mr = 0u, ml = 0u;
+  if (row >= 0) {
+    row_sides(rv, !use_r ? -f_inf() : (exact ? f_inf() : short_max(r.t[kR])),
+              !use_l ? -f_inf() : (exact ? f_inf() : short_max(r.t[kL])), S.ctrl->eps_feas,
+              inf_flag);
+    if (rv.act) {
+      if (use_r)
+        mr = short_survivors(r.t[kR], len, d_isfinite(rv.rhs), rv.mininf, r.kinf[kR], rv.thr_r,
+                             exact);
+      if (use_l)
+        ml = short_survivors(r.t[kL], len, d_isfinite(rv.lhs), rv.maxinf, r.kinf[kL], rv.thr_l,
+                             exact);
+    }
+  }
+  uint32_t m = mr | ml;
+  int pos = warp_reserve<4>(__popc(m), &S.ctrl->qcount);
+  if (m == 0u) return;
+  RowSum rs;
+  rs.minfin = rv.minfin;
+  rs.maxfin = rv.maxfin;
+  rs.mininf = rv.mininf;
+  rs.maxinf = rv.maxinf;
+  S.rowsum[c] = rs;
+  for (; m != 0u; m &= m - 1u, ++pos) {
+    const int k = __ffs(m) - 1;
+    CandEntry e;
+    e.off = (uint32_t)(elem0 + k * kSliceW);
+    e.cs = ((uint32_t)c << 2) | ((mr >> k) & 1u) | (((ml >> k) & 1u) << 1);
+    S.queue[pos] = e;
+  }
+}
+
+template <bool kMulti>
+__device__ __forceinline__ void short_slice(const DevMatrix &M, const DevState &S, int slice) {
+  const int lane = threadIdx.x & 31;
+  const int64_t c = (int64_t)slice * kSliceW + lane;
+  const int32_t lenf = M.chunk_len[c];
+  int32_t len = lenf & kLenMask;
+  int32_t row = M.chunk_row[c];
+  int32_t *inf_flag = &S.ctrl->infeasible;
+  if (kMulti && row >= 0) {  // a stopped problem's rows do nothing
+    const int32_t inst = S.I.slot_inst[c];
+    if (S.I.done[inst]) {
+      row = -1;
+      len = 0;
+    } else {
+      inf_flag = &S.I.infeasible[inst];
+    }
+  }
+  const double2 sd = (row >= 0) ? S.side[c] : make_double2(0.0, 0.0);
+  const bool need_min = __any_sync(kFull, row >= 0 && d_isfinite(sd.y));
+  const bool need_max = __any_sync(kFull, row >= 0 && d_isfinite(sd.x));
+  const int64_t elem0 = M.slice_off[slice] + lane;
+  const bool exact = (lenf & kExactFlag) != 0;
+  if (need_min && need_max)
+    short_rows<2>(M, S, c, elem0, len, row, exact, sd, true, inf_flag);
+  else
+    short_rows<1>(M, S, c, elem0, len, row, exact, sd, need_min, inf_flag);
+}
+
 template <bool kMulti, int kRoundWarps, bool kVal8>
-__global__ void __launch_bounds__(kRoundWarps * 32,
-                                  (kMulti ? kRoundWarpsPerSMMulti : kRoundWarpsPerSM) / kRoundWarps)
+__global__ void __launch_bounds__(kRoundWarps * 32, kRoundWarpsPerSM / kRoundWarps)
 k_round(DevMatrix M, DevState S) {
   if (S.ctrl->err) return;
   const int slice = blockIdx.x * kRoundWarps + (threadIdx.x >> 5);
   if (slice >= M.nslices) return;  // warp-uniform
-  round_slice<kMulti, kVal8, kMulti ? kGroupWide : kGroup>(M, S, slice);
+  if (!kVal8 && slice >= M.short0) short_slice<kMulti>(M, S, slice);
+  else round_slice<kMulti, kVal8>(M, S, slice);
 }
 
 // ------------------------------------------------------------- k_floor --
@@ -752,10 +845,10 @@ k_persistent(DevMatrix M, DevState S, const uint8_t *vartype) {
   for (;;) {
     if (M.val8)
       for (int sl = gw; sl < M.nslices; sl += nw)
-        round_slice<kMulti, true, kGroupWide, true>(M, S, sl);
+        round_slice<kMulti, true, true>(M, S, sl);
     else
       for (int sl = gw; sl < M.nslices; sl += nw)
-        round_slice<kMulti, false, kGroupWide, true>(M, S, sl);
+        round_slice<kMulti, false, true>(M, S, sl);
     if (!grid_sync(S, lim)) return;
     if (M.nsplit_rows > 0) {
       for (int w = gw; w < M.nsplit_rows; w += nw) combine_rows<kMulti>(M, S, w);

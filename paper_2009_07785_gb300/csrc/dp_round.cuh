@@ -24,21 +24,145 @@ __device__ __forceinline__ Top2 top2_init() {
   return t;
 }
 
-// Reserves c (0..7) consecutive queue entries per lane with one atomic per
-// warp (all 32 lanes call): the lanes' offsets come from three ballots of
-// the bits of c, not from a shuffle scan.  Returns the lane's first entry
+// ---- rows of at most kMax nonzeros ----
+//
+// A lane keeps the screen values of such a row in registers (the loops over
+// its slots are unrolled), so that the survivors are known from the row's
+// thresholds without another pass over its nonzeros, and the running top-2 of
+// the longer rows is not needed either.
+// What the unrolled pass leaves: kSides = 1: one side's sums and values,
+// kSides = 2: the minimum activity first, then the maximum.
+template <int kSides, int kMax>
+struct ShortAct {
+  double fin[kSides];
+  int32_t ninf[kSides], kinf[kSides];
+  float t[kSides][kMax];
+};
+
+// Activity sums, infinity counts and screen values of the lane's row (len <=
+// kMax slots from elem0, stride kSliceW; 0 for none).  kSides = 1:
+// `right` selects the minimum activity (the right-hand side's), else the
+// maximum.  rec(j, L, U, WU, WL) loads a record.  The sums are one FMA chain
+// in CSR order.  All 32 lanes call.
+template <int kSides, int kMax, class Rec>
+__device__ __forceinline__ void short_activity(const DevMatrix &M, int64_t elem0, int32_t len,
+                                               bool right, Rec rec,
+                                               ShortAct<kSides, kMax> &r) {
+  constexpr int kG = 4;
+  const int maxlen = __reduce_max_sync(kFull, len);
+  const double *vp = M.val + elem0;
+  const int32_t *cp = M.col + elem0;
+#pragma unroll
+  for (int s = 0; s < kSides; ++s) {
+    r.fin[s] = 0.0;
+    r.ninf[s] = r.kinf[s] = 0;
+  }
+  double an[kG];
+  int32_t jn[kG];
+#pragma unroll
+  for (int u = 0; u < kG; ++u) {
+    an[u] = 1.0;
+    jn[u] = 0;
+    if (u < len) {
+      an[u] = __ldcs(vp + u * kSliceW);
+      jn[u] = __ldcs(cp + u * kSliceW);
+    }
+  }
+#pragma unroll
+  for (int g = 0; g < kMax / kG; ++g) {
+    if (g > 0 && g * kG >= maxlen) {  // warp-uniform
+#pragma unroll
+      for (int u = 0; u < kG; ++u)
+#pragma unroll
+        for (int s = 0; s < kSides; ++s) r.t[s][g * kG + u] = -f_inf();
+      continue;
+    }
+    double a[kG], L[kG], U[kG];
+    float WU[kG], WL[kG];
+#pragma unroll
+    for (int u = 0; u < kG; ++u) {
+      a[u] = an[u];
+      L[u] = U[u] = 0.0;
+      WU[u] = WL[u] = 0.0f;
+      if (g * kG + u < len) rec(jn[u], L[u], U[u], WU[u], WL[u]);
+    }
+    if ((g + 1) * kG < kMax && (g + 1) * kG < maxlen) {
+#pragma unroll
+      for (int u = 0; u < kG; ++u) {
+        an[u] = 1.0;
+        jn[u] = 0;
+        if ((g + 1) * kG + u < len) {
+          an[u] = __ldcs(vp + ((g + 1) * kG + u) * kSliceW);
+          jn[u] = __ldcs(cp + ((g + 1) * kG + u) * kSliceW);
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kG; ++u) {
+      const int k = g * kG + u;
+      const float au = absup_fast(a[u]), ad = absdn_fast(a[u]);
+#pragma unroll
+      for (int s = 0; s < kSides; ++s) {
+        const bool low = d_pos(a[u]) == (kSides == 2 ? s == 0 : right);
+        const double b = low ? L[u] : U[u];
+        const bool inf = d_isinf(b);
+        const float t = screen_prod(au, ad, low ? WU[u] : WL[u]);
+        r.t[s][k] = k < len ? t : -f_inf();
+        if (k < len) {
+          r.ninf[s] += inf;
+          if (inf) r.kinf[s] = k;
+          r.fin[s] = fma(a[u], inf ? 0.0 : b, r.fin[s]);
+        }
+      }
+    }
+  }
+}
+
+// The largest screen value of a side.
+template <int kMax>
+__device__ __forceinline__ float short_max(const float (&t)[kMax]) {
+  float m = t[0];
+#pragma unroll
+  for (int k = 1; k < kMax; ++k) m = fmaxf(m, t[k]);
+  return m;
+}
+
+// The slots of a row that survive one side's screen (bit k: slot k); `fin`:
+// the side is finite.
+template <int kMax>
+__device__ __forceinline__ uint32_t short_survivors(const float (&t)[kMax], int32_t len,
+                                                    bool fin, int32_t ninf, int32_t kinf,
+                                                    float thr, bool exact) {
+  if (!fin || ninf > 1) return 0u;
+  if (ninf == 1) return 1u << kinf;
+  const uint32_t all = (1u << len) - 1u;
+  if (exact) return f_inf() > thr ? all : 0u;
+  uint32_t m = 0u;
+#pragma unroll
+  for (int k = 0; k < kMax; ++k)
+    if (t[k] > thr) m |= 1u << k;
+  return m & all;
+}
+
+// Reserves c (0..15) consecutive queue entries per lane with one atomic per
+// warp (all 32 lanes call): the lanes' offsets come from ballots of the bits
+// of c (kBits of them), not from a shuffle scan.  Returns the lane's first entry
 // (meaningless when c = 0).
+template <int kBits = 3>
 __device__ __forceinline__ int warp_reserve(int c, int32_t *counter) {
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
-  const unsigned b0 = __ballot_sync(kFull, c & 1), b1 = __ballot_sync(kFull, c & 2),
-                 b2 = __ballot_sync(kFull, c & 4);
-  const int total = __popc(b0) + 2 * __popc(b1) + 4 * __popc(b2);
+  int total = 0, before = 0;
+#pragma unroll
+  for (int k = 0; k < kBits; ++k) {
+    const unsigned b = __ballot_sync(kFull, c & (1 << k));
+    total += __popc(b) << k;
+    before += __popc(b & lt) << k;
+  }
   if (total == 0) return 0;
   int base = 0;
   if (lane == 0) base = atomicAdd(counter, total);
-  base = __shfl_sync(kFull, base, 0);
-  return base + __popc(b0 & lt) + 2 * __popc(b1 & lt) + 4 * __popc(b2 & lt);
+  return __shfl_sync(kFull, base, 0) + before;
 }
 
 // Queues nonzeros of the lanes' chunks whose candidates survive the screen.
