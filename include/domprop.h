@@ -469,7 +469,10 @@ int dp_propagate_noalloc(int device, void *cuda_stream, int32_t m, int32_t n,
  * indices node + j*nodes stay below 2^30); 32 nodes share each warp, so
  * counts that are multiples of 32 use the device best.  The first call
  * allocates a workspace of about 80 bytes per (variable, node) pair kept
- * with the matrix (freed by dp_matrix_free); host inputs are staged.
+ * with the matrix (freed by dp_matrix_free); host inputs are staged.  Few
+ * nodes of a small matrix run on a thread block cluster each instead, with a
+ * workspace of about 50 bytes per variable and cluster; the results are the
+ * same.
  * Returns DP_OK, DP_CAP_HIT (some node hit the cap), DP_ERR_INVALID_ARG,
  * DP_ERR_NAN_INPUT (any node), DP_ERR_OOM or DP_ERR_CUDA.
  */

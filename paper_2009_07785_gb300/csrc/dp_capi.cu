@@ -85,6 +85,44 @@ int upload(dp_matrix *mat, const std::vector<T> &v, const T **out, cudaStream_t 
 
 using dp::is_device_ptr;
 
+// Where a team (dp_team.cu) takes a problem instead of the graph's kernels or
+// the batched ones.  A team's rounds cost less (a cluster barrier instead of
+// three to five kernels) and its marking skips unchanged rows, but it has 16
+// blocks at most.  Measured in us per call (graph or batch / team):
+//   one problem:  short rows 60k nonzeros 460 / 384, 179k 571 / 797;
+//                 irregular 60k 1112 / 634, 235k 1397 / 1275, 704k 2211 / 3790;
+//                 mixed 25k 1796 / 866, 126k 1750 / 1327, 378k 2187 / 2748
+//   nodes:        irregular 60k nonzeros, 33 nodes 1547 / 1073, 128 nodes
+//                 1974 / 2136; 235k, 8 nodes 2859 / 1474, 33 nodes 3783 / 2896,
+//                 128 nodes 5462 / 8902; 2.0M, 1 node 5717 / 6534;
+//                 short 24k, 128 nodes 1072 / 915, 256 nodes 1453 / 1494
+//   sets:         12 problems of up to 29k nonzeros 2855 / 842; 64 of up to
+//                 1.7M 8331 / 22885
+constexpr int64_t kTeamNnz = 100000;       // a single problem, or a set's largest
+constexpr int64_t kTeamSetNnz = 4000000;   // a whole set
+constexpr int64_t kTeamNodeNnz = 300000;   // the matrix of a node batch
+constexpr int64_t kTeamNodeWork = 6000000; // its nonzeros times nodes
+constexpr int kTeamWarps = 8;  // warps per block of a team
+
+// Blocks of a team, a power of two: no more than give every slice a warp and
+// all `count` teams room at once.
+int team_size(const dp_ctx *ctx, int32_t nslices, int32_t count) {
+  int k = 4;
+  while (k > 0 && ((1 << k) > 2 * ((nslices + kTeamWarps - 1) / kTeamWarps) - 1 ||
+                   ctx->teams_of[k] < count))
+    --k;
+  return k;  // log2
+}
+
+// The parameters of a call.
+void team_params(dp::TeamArgs &A, const dp_params &p) {
+  A.max_rounds = p.max_rounds;
+  A.eps_int = p.eps_int;
+  A.tau_rel = p.tau_rel;
+  A.eps_feas = p.eps_feas;
+  A.inf_thr = p.inf_threshold;
+}
+
 // Makes a round-loop graph: one WHILE node whose body is the kernels that
 // `body(handle, stream)` launches; the condition starts at 1 on every launch
 // and the last kernel of the body sets it on the device.
@@ -244,6 +282,7 @@ int dp_create(dp_ctx **out, int device, void *cuda_stream) {
     delete ctx;
     return DP_ERR_CUDA;
   }
+  for (int k = 0; k < 5; ++k) ctx->teams_of[k] = dp::cluster_teams_resident(1 << k);
   if (cuda_stream) {
     ctx->stream = static_cast<cudaStream_t>(cuda_stream);
   } else {
@@ -280,6 +319,17 @@ void free_batch(BatchWs *b) {
   if (b->h_nodes) cudaFreeHost(b->h_nodes);
   delete b;
 }
+
+void free_teams(TeamWs *t) {
+  if (!t) return;
+  for (void *p : t->allocs) dp::dev_free(p);
+  dp::dev_free(t->st_lb);
+  dp::dev_free(t->st_ub);
+  dp::dev_free(t->out_lb);
+  dp::dev_free(t->out_ub);
+  if (t->h_res) cudaFreeHost(t->h_res);
+  delete t;
+}
 }  // namespace
 
 void dp_matrix_free(dp_matrix *mat) {
@@ -287,7 +337,9 @@ void dp_matrix_free(dp_matrix *mat) {
   cudaSetDevice(mat->ctx->device);
   cudaStreamSynchronize(mat->ctx->stream);
   free_batch(mat->batch);
+  free_teams(mat->teams);
   if (mat->h_inst) cudaFreeHost(mat->h_inst);
+  if (mat->h_res) cudaFreeHost(mat->h_res);
   if (mat->exec) cudaGraphExecDestroy(mat->exec);
   if (mat->graph) cudaGraphDestroy(mat->graph);
   for (void *p : mat->allocs) dp::dev_free(p);
@@ -307,21 +359,14 @@ int dp_matrix_load(dp_ctx *ctx, int32_t m, int32_t n, int64_t nnz,
 
 namespace {
 
-// Loads a matrix; with row_off/var_off (count+1 offsets each) it is the
-// block-diagonal union of `count` independent problems; with merge_ipt > 0
-// it gets the merge-path layout with that many items per segment.
-int load_impl(dp_ctx *ctx, int32_t m, int32_t n, int64_t nnz, const int64_t *row_ptr,
-              const int32_t *col_idx, const double *val, int32_t chunk, const double *lhs,
-              const double *rhs, const std::vector<int32_t> *row_off,
-              const std::vector<int32_t> *var_off, dp_matrix **out, int32_t merge_ipt = 0) {
-  if (!ctx || !out) return DP_ERR_INVALID_ARG;
-  *out = nullptr;
-  if ((lhs == nullptr) != (rhs == nullptr)) return DP_ERR_INVALID_ARG;
-  dp::HostLayout H;
-  int rc = merge_ipt > 0
-               ? dp::build_merge_layout(m, n, nnz, row_ptr, col_idx, val, merge_ipt, lhs, rhs, H)
-               : dp::build_layout(m, n, nnz, row_ptr, col_idx, val, chunk, lhs, rhs, H);
-  if (rc) return rc;
+// Loads a matrix from its host layout; with row_off/var_off (count+1 offsets
+// each) it is the block-diagonal union of `count` independent problems, whose
+// `views` come largest first.
+int load_layout(dp_ctx *ctx, dp::HostLayout &H, const std::vector<int32_t> *row_off,
+                const std::vector<int32_t> *var_off, const std::vector<dp::TeamView> *views,
+                dp_matrix **out) {
+  const int32_t m = H.m, n = H.n;
+  const int64_t nnz = H.nnz;
   CUDA_TRY(cudaSetDevice(ctx->device));
   dp_matrix *mat = new (std::nothrow) dp_matrix();
   if (!mat) return DP_ERR_OOM;
@@ -336,9 +381,9 @@ int load_impl(dp_ctx *ctx, int32_t m, int32_t n, int64_t nnz, const int64_t *row
   M.nslices_split = H.nslices_split;
   M.nsplit_rows = H.nsplit_rows;
   M.round_warps = 8;
-  // whole rows are sorted by length, longest first
+  // a single problem's whole rows are sorted by length, longest first
   M.short0 = H.nslices;
-  while (H.layout == dp::kLayoutEll && M.short0 > H.nslices_split &&
+  while (H.layout == dp::kLayoutEll && !row_off && M.short0 > H.nslices_split &&
          H.slice_len[(size_t)M.short0 - 1] <= dp::kShortRow)
     --M.short0;
   M.layout = H.layout;
@@ -346,6 +391,12 @@ int load_impl(dp_ctx *ctx, int32_t m, int32_t n, int64_t nnz, const int64_t *row
   M.mp_nseg = H.mp_nseg;
   M.mp_nlong = H.mp_nlong;
   M.mp_npiece = (int32_t)H.mp_piece.size();
+  if (H.layout == dp::kLayoutEll) {  // both kinds of slices are sorted, longest first
+    auto is_long = [&](int32_t q) { return H.slice_len[(size_t)q] >= dp::kLongSlots; };
+    while (M.long_split < M.nslices_split && is_long(M.long_split)) ++M.long_split;
+    while (M.nslices_split + M.long_whole < M.nslices && is_long(M.nslices_split + M.long_whole))
+      ++M.long_whole;
+  }
   mat->padded = (int64_t)H.val.size();
 #define TRY(x)                 \
   do {                         \
@@ -393,8 +444,33 @@ int load_impl(dp_ctx *ctx, int32_t m, int32_t n, int64_t nnz, const int64_t *row
   TRY(dev_alloc(mat, &S.rowsum, (size_t)H.nslices * dp::kSliceW));
   TRY(dev_alloc(mat, &S.side, (size_t)H.nslices * dp::kSliceW));
   TRY(dev_alloc(mat, &S.ctrl, 1));
-  TRY(dev_alloc(mat, &S.dirty, ((size_t)n + 31) / 32));  // dirty bitmap
+  // dirty bitmap (a set's problems start at words of their own when teams run)
+  TRY(dev_alloc(mat, &S.dirty, ((size_t)n + 31) / 32 + (views ? views->size() : 0)));
   TRY(dev_alloc(mat, &S.bar, 2));
+  if (H.layout == dp::kLayoutEll) {
+    int32_t *ptr = nullptr, *slot = nullptr;
+    TRY(dev_alloc(mat, &ptr, (size_t)n + 1));
+    TRY(dev_alloc(mat, &slot, (size_t)nnz));
+    const size_t nflags = views ? views->size() : 1;
+    TRY(dev_alloc(mat, &mat->team_flags, nflags));
+    TRY(dev_alloc(mat, &mat->team_mask, 2 * (size_t)H.nslices));
+    TRY(dev_alloc(mat, &mat->team_touch, (size_t)H.nsplit_rows));
+    // the counts' scratch: the keys are not in use yet
+    if (dp::launch_columns(M, reinterpret_cast<int32_t *>(S.keys), ptr, slot, ctx->num_sms, st) !=
+            cudaSuccess ||
+        cudaMemsetAsync(mat->team_flags, 0, sizeof(dp::TeamFlags) * nflags, st) != cudaSuccess) {
+      cudaGetLastError();
+      dp_matrix_free(mat);
+      return DP_ERR_CUDA;
+    }
+    M.col_ptr = ptr;
+    M.col_slot = slot;
+    if (cudaMallocHost(&mat->h_res, sizeof(int4) * nflags) != cudaSuccess) {
+      cudaGetLastError();
+      dp_matrix_free(mat);
+      return DP_ERR_OOM;
+    }
+  }
   TRY(dev_alloc(mat, &mat->vt_ws, (size_t)n));
   TRY(dev_alloc(mat, &mat->st_lb, (size_t)n));
   TRY(dev_alloc(mat, &mat->st_ub, (size_t)n));
@@ -424,6 +500,10 @@ int load_impl(dp_ctx *ctx, int32_t m, int32_t n, int64_t nnz, const int64_t *row
     TRY(dev_alloc(mat, &S.I.status, (size_t)count));
     S.I.ninst = count;
     mat->ninst = count;
+    const dp::TeamView *dv = nullptr;
+    TRY(upload(mat, *views, &dv, st));
+    mat->d_views = const_cast<dp::TeamView *>(dv);
+    TRY(dev_alloc(mat, &mat->team_next, 1));
     mat->row_off = *row_off;
     mat->var_off = *var_off;
     if (cudaMallocHost(&mat->h_inst, sizeof(int32_t) * 3 * (size_t)count) != cudaSuccess) {
@@ -443,6 +523,22 @@ int load_impl(dp_ctx *ctx, int32_t m, int32_t n, int64_t nnz, const int64_t *row
   return DP_OK;
 }
 
+// Loads one matrix; with merge_ipt > 0 it gets the merge-path layout with
+// that many items per segment.
+int load_impl(dp_ctx *ctx, int32_t m, int32_t n, int64_t nnz, const int64_t *row_ptr,
+              const int32_t *col_idx, const double *val, int32_t chunk, const double *lhs,
+              const double *rhs, dp_matrix **out, int32_t merge_ipt = 0) {
+  if (!ctx || !out) return DP_ERR_INVALID_ARG;
+  *out = nullptr;
+  if ((lhs == nullptr) != (rhs == nullptr)) return DP_ERR_INVALID_ARG;
+  dp::HostLayout H;
+  int rc = merge_ipt > 0
+               ? dp::build_merge_layout(m, n, nnz, row_ptr, col_idx, val, merge_ipt, lhs, rhs, H)
+               : dp::build_layout(m, n, nnz, row_ptr, col_idx, val, chunk, lhs, rhs, H);
+  if (rc) return rc;
+  return load_layout(ctx, H, nullptr, nullptr, nullptr, out);
+}
+
 }  // namespace
 
 extern "C" {
@@ -452,8 +548,7 @@ int dp_matrix_load_sides(dp_ctx *ctx, int32_t m, int32_t n, int64_t nnz,
                          int32_t chunk, const double *lhs, const double *rhs,
                          dp_matrix **out) {
   dp::TraceRange trace_range("dp_matrix_load_sides");
-  return load_impl(ctx, m, n, nnz, row_ptr, col_idx, val, chunk, lhs, rhs, nullptr, nullptr,
-                   out);
+  return load_impl(ctx, m, n, nnz, row_ptr, col_idx, val, chunk, lhs, rhs, out);
 }
 
 int dp_matrix_load_merge(dp_ctx *ctx, int32_t m, int32_t n, int64_t nnz,
@@ -465,8 +560,7 @@ int dp_matrix_load_merge(dp_ctx *ctx, int32_t m, int32_t n, int64_t nnz,
     if (out) *out = nullptr;
     return DP_ERR_INVALID_ARG;
   }
-  return load_impl(ctx, m, n, nnz, row_ptr, col_idx, val, 0, lhs, rhs, nullptr, nullptr, out,
-                   items_per_thread);
+  return load_impl(ctx, m, n, nnz, row_ptr, col_idx, val, 0, lhs, rhs, out, items_per_thread);
 }
 
 int dp_matrix_load_set(dp_ctx *ctx, int32_t count, const int32_t *m, const int32_t *n,
@@ -490,39 +584,22 @@ int dp_matrix_load_set(dp_ctx *ctx, int32_t count, const int32_t *m, const int32
     row_off.push_back((int32_t)mt);
     var_off.push_back((int32_t)nt);
   }
-  std::vector<int64_t> rp;
-  std::vector<int32_t> col;
-  std::vector<double> vv, sl, sr;
-  try {
-    rp.reserve((size_t)mt + 1);
-    col.reserve((size_t)nzt);
-    vv.reserve((size_t)nzt);
-    rp.push_back(0);
-    for (int32_t k = 0; k < count; ++k) {
-      const int64_t base = rp.back();
-      for (int32_t i = 0; i < m[k]; ++i) rp.push_back(base + row_ptr[k][i + 1]);
-      const int64_t nz = m[k] > 0 ? row_ptr[k][m[k]] : 0;
-      if (m[k] > 0 && row_ptr[k][0] != 0) return DP_ERR_BAD_CSR;
-      if (nz > 0 && (!col_idx[k] || !val[k])) return DP_ERR_INVALID_ARG;
-      for (int64_t q = 0; q < nz; ++q) {
-        const int32_t c = col_idx[k][q];
-        if (c < 0 || c >= n[k]) return DP_ERR_BAD_CSR;
-        col.push_back(c + var_off[(size_t)k]);
-        vv.push_back(val[k][q]);
-      }
-      if (lhs) {
-        for (int32_t i = 0; i < m[k]; ++i) {
-          sl.push_back(lhs[k][i]);
-          sr.push_back(rhs[k][i]);
-        }
-      }
-    }
-  } catch (const std::bad_alloc &) {
-    return DP_ERR_OOM;
+  for (int32_t k = 0; k < count; ++k) {
+    if (m[k] > 0 && row_ptr[k][0] != 0) return DP_ERR_BAD_CSR;
+    if (m[k] > 0 && row_ptr[k][m[k]] > 0 && (!col_idx[k] || !val[k])) return DP_ERR_INVALID_ARG;
   }
-  return load_impl(ctx, (int32_t)mt, (int32_t)nt, nzt, rp.data(), col.data(), vv.data(), chunk,
-                   lhs ? sl.data() : nullptr, lhs ? sr.data() : nullptr, &row_off, &var_off,
-                   out);
+  dp::HostLayout H;
+  std::vector<dp::TeamView> views;
+  const int rc = dp::build_set_layout(count, m, n, row_ptr, col_idx, val, chunk, lhs, rhs, H, views);
+  if (rc) return rc;
+  dp_matrix *set = nullptr;
+  const int lrc = load_layout(ctx, H, &row_off, &var_off, &views, &set);
+  if (lrc) return lrc;
+  const dp::TeamView &V = views.front();
+  set->largest = m[V.id] > 0 ? row_ptr[V.id][m[V.id]] : 0;
+  set->view_slices = (V.split1 - V.split0) + (V.whole1 - V.whole0);
+  *out = set;
+  return DP_OK;
 }
 
 int dp_matrix_set_launch(dp_matrix *mat, int32_t round_warps) {
@@ -615,25 +692,40 @@ int dp_matrix_access_floor(dp_ctx *ctx, const dp_matrix *mat, int32_t reps, floa
 
 namespace {
 
+// One call's inputs on the device.
+struct DevInputs {
+  const double *lb, *ub, *lhs, *rhs;
+  const uint8_t *vt;
+};
+
+// Device pointers are read in place, host pointers staged.
+int stage_inputs(dp_ctx *ctx, dp_matrix *mat, const double *lb, const double *ub,
+                 const uint8_t *vartype, const double *lhs, const double *rhs, DevInputs *d) {
+  const int32_t m = mat->M.m, n = mat->M.n;
+  CUDA_TRY(cudaSetDevice(ctx->device));
+  cudaStream_t st = ctx->stream;
+  *d = {lb, ub, lhs, rhs, vartype};
+  if (n > 0) {
+    if (!is_device_ptr(lb)) { CUDA_TRY(cudaMemcpyAsync(mat->st_lb, lb, 8 * (size_t)n, cudaMemcpyDefault, st)); d->lb = mat->st_lb; }
+    if (!is_device_ptr(ub)) { CUDA_TRY(cudaMemcpyAsync(mat->st_ub, ub, 8 * (size_t)n, cudaMemcpyDefault, st)); d->ub = mat->st_ub; }
+    if (!is_device_ptr(vartype)) { CUDA_TRY(cudaMemcpyAsync(mat->st_vt, vartype, (size_t)n, cudaMemcpyDefault, st)); d->vt = mat->st_vt; }
+  }
+  if (m > 0) {
+    if (!is_device_ptr(lhs)) { CUDA_TRY(cudaMemcpyAsync(mat->st_lhs, lhs, 8 * (size_t)m, cudaMemcpyDefault, st)); d->lhs = mat->st_lhs; }
+    if (!is_device_ptr(rhs)) { CUDA_TRY(cudaMemcpyAsync(mat->st_rhs, rhs, 8 * (size_t)m, cudaMemcpyDefault, st)); d->rhs = mat->st_rhs; }
+  }
+  return DP_OK;
+}
+
 // Stages inputs, writes the control block and runs the prologue.
 int begin_call(dp_ctx *ctx, dp_matrix *mat, const double *lb, const double *ub,
                const uint8_t *vartype, const double *lhs, const double *rhs,
                const dp_params &p) {
   const int32_t m = mat->M.m, n = mat->M.n;
-  CUDA_TRY(cudaSetDevice(ctx->device));
+  DevInputs d;
+  int rc = stage_inputs(ctx, mat, lb, ub, vartype, lhs, rhs, &d);
+  if (rc) return rc;
   cudaStream_t st = ctx->stream;
-  // inputs: device pointers are read in place, host pointers staged
-  const double *d_lb = lb, *d_ub = ub, *d_lhs = lhs, *d_rhs = rhs;
-  const uint8_t *d_vt = vartype;
-  if (n > 0) {
-    if (!is_device_ptr(lb)) { CUDA_TRY(cudaMemcpyAsync(mat->st_lb, lb, 8 * (size_t)n, cudaMemcpyDefault, st)); d_lb = mat->st_lb; }
-    if (!is_device_ptr(ub)) { CUDA_TRY(cudaMemcpyAsync(mat->st_ub, ub, 8 * (size_t)n, cudaMemcpyDefault, st)); d_ub = mat->st_ub; }
-    if (!is_device_ptr(vartype)) { CUDA_TRY(cudaMemcpyAsync(mat->st_vt, vartype, (size_t)n, cudaMemcpyDefault, st)); d_vt = mat->st_vt; }
-  }
-  if (m > 0) {
-    if (!is_device_ptr(lhs)) { CUDA_TRY(cudaMemcpyAsync(mat->st_lhs, lhs, 8 * (size_t)m, cudaMemcpyDefault, st)); d_lhs = mat->st_lhs; }
-    if (!is_device_ptr(rhs)) { CUDA_TRY(cudaMemcpyAsync(mat->st_rhs, rhs, 8 * (size_t)m, cudaMemcpyDefault, st)); d_rhs = mat->st_rhs; }
-  }
   dp::Ctrl *hc = ctx->h_ctrl;
   std::memset(hc, 0, sizeof(*hc));
   hc->max_rounds = p.max_rounds;
@@ -643,7 +735,7 @@ int begin_call(dp_ctx *ctx, dp_matrix *mat, const double *lb, const double *ub,
   hc->inf_thr = p.inf_threshold;
   hc->wait_limit = ctx->wait_limit;
   CUDA_TRY(cudaMemcpyAsync(mat->S.ctrl, hc, sizeof(*hc), cudaMemcpyHostToDevice, st));
-  CUDA_TRY(dp::launch_prologue(mat->M, mat->S, mat->vt_ws, m, n, d_lb, d_ub, d_vt, d_lhs, d_rhs,
+  CUDA_TRY(dp::launch_prologue(mat->M, mat->S, mat->vt_ws, m, n, d.lb, d.ub, d.vt, d.lhs, d.rhs,
                                p.eps_int, p.tau_rel, p.inf_threshold, ctx->num_sms, st));
   return DP_OK;
 }
@@ -689,6 +781,57 @@ int check_call(dp_ctx *ctx, const dp_matrix *mat, const double *lb, const double
   return DP_OK;
 }
 
+// Whether teams, one per problem, beat the graph over the union.
+bool teams_for_set(const dp_matrix *set) {
+  return set->h_res && set->largest <= kTeamNnz && set->M.nnz <= kTeamSetNnz;
+}
+
+// The whole propagation of one small problem by one team, or of every problem
+// of a set by a team each; results in mat->h_res.
+int team_call(dp_ctx *ctx, dp_matrix *mat, const double *lb, const double *ub,
+              const uint8_t *vartype, const double *lhs, const double *rhs, const dp_params &p,
+              double *lb_out, double *ub_out) {
+  const size_t n = (size_t)mat->M.n;
+  DevInputs d;
+  int rc = stage_inputs(ctx, mat, lb, ub, vartype, lhs, rhs, &d);
+  if (rc) return rc;
+  cudaStream_t st = ctx->stream;
+  const bool dl = n == 0 || is_device_ptr(lb_out), du = n == 0 || is_device_ptr(ub_out);
+  const int32_t count = mat->ninst > 0 ? mat->ninst : 1;
+  dp::TeamArgs A{};
+  A.M = mat->M;
+  A.rec = mat->S.rec;
+  A.keys = reinterpret_cast<longlong2 *>(mat->S.keys);
+  A.dirty = mat->S.dirty;
+  A.mask = mat->team_mask;
+  A.touch = mat->team_touch;
+  A.part = mat->S.part;
+  A.rowtot = mat->S.rowtot;
+  A.flags = mat->team_flags;
+  A.side = mat->S.side;
+  A.views = mat->d_views;
+  A.next = mat->team_next;
+  A.lb = d.lb;
+  A.ub = d.ub;
+  A.lhs = d.lhs;
+  A.rhs = d.rhs;
+  A.vt = d.vt;
+  A.lb_out = dl ? lb_out : mat->out_lb;
+  A.ub_out = du ? ub_out : mat->out_ub;
+  A.res = mat->h_res;
+  A.count = count;
+  team_params(A, p);
+  const int k = team_size(ctx, mat->ninst > 0 ? mat->view_slices : A.M.nslices, count);
+  const int32_t teams = count < ctx->teams_of[k] ? count : ctx->teams_of[k];
+  CUDA_TRY(dp::launch_cluster_teams(A, teams, 1 << k, ctx->num_sms, st));
+  if (!dl) CUDA_TRY(cudaMemcpyAsync(lb_out, A.lb_out, 8 * n, cudaMemcpyDefault, st));
+  if (!du) CUDA_TRY(cudaMemcpyAsync(ub_out, A.ub_out, 8 * n, cudaMemcpyDefault, st));
+  CUDA_TRY(cudaStreamSynchronize(st));
+  for (int32_t i = 0; i < count; ++i)
+    if (mat->h_res[i].w) return mat->h_res[i].w;
+  return DP_OK;
+}
+
 }  // namespace
 
 extern "C" {
@@ -703,6 +846,14 @@ int dp_propagate(dp_ctx *ctx, const dp_matrix *cmat, const double *lb,
                       infeasible, rounds, &p);
   if (rc) return rc;
   dp_matrix *mat = const_cast<dp_matrix *>(cmat);
+  if (mat->h_res && mat->ninst == 0 && !mat->M.val8 && mat->M.nnz <= kTeamNnz &&
+      ctx->teams_of[0] > 0) {
+    rc = team_call(ctx, mat, lb, ub, vartype, lhs, rhs, p, lb_out, ub_out);
+    if (rc) return rc;
+    *infeasible = mat->h_res->x;
+    *rounds = mat->h_res->y;
+    return mat->h_res->z ? DP_CAP_HIT : DP_OK;
+  }
   rc = begin_call(ctx, mat, lb, ub, vartype, lhs, rhs, p);
   if (rc) return rc;
   if (p.max_rounds > 0) CUDA_TRY(cudaGraphLaunch(mat->exec, ctx->stream));
@@ -756,6 +907,18 @@ int set_call(dp_ctx *ctx, const dp_matrix *cset, const double *lb, const double 
       return DP_ERR_CUDA;
   }
   dp_matrix *set = const_cast<dp_matrix *>(cset);
+  if (!persistent && !set->M.val8 && ctx->teams_of[0] > 0 && teams_for_set(set)) {
+    rc = team_call(ctx, set, lb, ub, vartype, lhs, rhs, p, lb_out, ub_out);
+    if (rc < 0) return rc;
+    bool cap = false;
+    for (int32_t k = 0; k < set->ninst; ++k) {
+      infeasible[k] = set->h_res[k].x;
+      rounds[k] = set->h_res[k].y;
+      if (status) status[k] = set->h_res[k].z;
+      cap |= set->h_res[k].z != 0;
+    }
+    return cap ? DP_CAP_HIT : DP_OK;
+  }
   rc = begin_call(ctx, set, lb, ub, vartype, lhs, rhs, p);
   if (rc) return rc;
   cudaStream_t st = ctx->stream;
@@ -1081,6 +1244,138 @@ int batch_hostloop(dp_matrix *mat, BatchWs *b, int32_t max_rounds, float *kernel
   return status;
 }
 
+// ---- nodes by teams ----
+
+// Makes (or reuses) the state of `slots` teams over the matrix.
+int ensure_teams(dp_matrix *mat, int32_t slots) {
+  if (mat->teams && mat->teams->slots >= slots) return DP_OK;
+  if (mat->teams) {
+    cudaStreamSynchronize(mat->ctx->stream);
+    free_teams(mat->teams);
+    mat->teams = nullptr;
+  }
+  TeamWs *t = new (std::nothrow) TeamWs();
+  if (!t) return DP_ERR_OOM;
+  const dp::DevMatrix &M = mat->M;
+  dp::TeamArgs &A = t->A;
+  A.M = M;
+  A.s_var = M.n;
+  A.s_dirty = ((int64_t)M.n + 31) / 32;
+  A.s_mask = 2 * (int64_t)M.nslices;
+  A.s_touch = M.nsplit_rows;
+  A.s_part = (int64_t)M.nslices_split * dp::kSliceW;
+  A.side = mat->S.side;
+  A.node_sums = 1;
+  const size_t k = (size_t)slots;
+  int rc;
+#define TTRY(x)                                                         do {                                                                    if ((rc = (x)) != DP_OK) {                                              free_teams(t);                                                        return rc;                                                          }                                                                   } while (0)
+  TTRY(dp::track_alloc(t->allocs, &A.rec, k * (size_t)A.s_var, nullptr));
+  TTRY(dp::track_alloc(t->allocs, &A.keys, k * (size_t)A.s_var, nullptr));
+  TTRY(dp::track_alloc(t->allocs, &A.dirty, k * (size_t)A.s_dirty, nullptr));
+  TTRY(dp::track_alloc(t->allocs, &A.mask, k * (size_t)A.s_mask, nullptr));
+  TTRY(dp::track_alloc(t->allocs, &A.touch, k * (size_t)A.s_touch, nullptr));
+  TTRY(dp::track_alloc(t->allocs, &A.part, k * (size_t)A.s_part, nullptr));
+  TTRY(dp::track_alloc(t->allocs, &A.rowtot, k * (size_t)A.s_touch, nullptr));
+  TTRY(dp::track_alloc(t->allocs, &A.flags, k, nullptr));
+  TTRY(dp::track_alloc(t->allocs, &A.next, 1, nullptr));
+#undef TTRY
+  if (cudaMemsetAsync(A.flags, 0, sizeof(dp::TeamFlags) * k, mat->ctx->stream) != cudaSuccess) {
+    cudaGetLastError();
+    free_teams(t);
+    return DP_ERR_CUDA;
+  }
+  t->slots = slots;
+  mat->teams = t;
+  return DP_OK;
+}
+
+// Device staging for `count` host bound vectors, grown when needed.
+int stage_teams(TeamWs *t, int64_t count, size_t n) {
+  if (t->stage_cap >= count) return DP_OK;
+  double **bufs[4] = {&t->st_lb, &t->st_ub, &t->out_lb, &t->out_ub};
+  t->stage_cap = 0;
+  for (double **b : bufs) {
+    dp::dev_free(*b);
+    *b = nullptr;
+    void *q = nullptr;
+    const cudaError_t e = dp::dev_malloc(&q, sizeof(double) * (size_t)count * (n > 0 ? n : 1));
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      return e == cudaErrorMemoryAllocation ? DP_ERR_OOM : DP_ERR_CUDA;
+    }
+    *b = static_cast<double *>(q);
+  }
+  t->stage_cap = count;
+  return DP_OK;
+}
+
+// dp_propagate_nodes with a team per node.
+int nodes_by_teams(dp_ctx *ctx, dp_matrix *mat, int32_t count, const double *lb, const double *ub,
+                   const uint8_t *vartype, const double *lhs, const double *rhs,
+                   const dp_params &p, double *lb_out, double *ub_out, int32_t *infeasible,
+                   int32_t *rounds, int32_t *status) {
+  const size_t n = (size_t)mat->M.n, m = (size_t)mat->M.m;
+  cudaStream_t st = ctx->stream;
+  const int k = team_size(ctx, mat->M.nslices, count);
+  const int32_t teams = count < ctx->teams_of[k] ? count : ctx->teams_of[k];
+  int rc = ensure_teams(mat, teams);
+  if (rc) return rc;
+  TeamWs *t = mat->teams;
+  const bool hl = n > 0 && !is_device_ptr(lb), hu = n > 0 && !is_device_ptr(ub);
+  const bool hol = n > 0 && !is_device_ptr(lb_out), hou = n > 0 && !is_device_ptr(ub_out);
+  if ((hl || hu || hol || hou) && (rc = stage_teams(t, count, n))) return rc;
+  if (t->res_cap < count) {
+    if (t->h_res) cudaFreeHost(t->h_res);
+    t->h_res = nullptr;
+    t->res_cap = 0;
+    if (cudaMallocHost(&t->h_res, sizeof(int4) * (size_t)count) != cudaSuccess) {
+      cudaGetLastError();
+      return DP_ERR_OOM;
+    }
+    t->res_cap = count;
+  }
+  const size_t bytes = sizeof(double) * (size_t)count * n;
+  dp::TeamArgs A = t->A;
+  A.lb = lb;
+  A.ub = ub;
+  A.vt = vartype;
+  A.lhs = lhs;
+  A.rhs = rhs;
+  if (hl) { CUDA_TRY(cudaMemcpyAsync(t->st_lb, lb, bytes, cudaMemcpyDefault, st)); A.lb = t->st_lb; }
+  if (hu) { CUDA_TRY(cudaMemcpyAsync(t->st_ub, ub, bytes, cudaMemcpyDefault, st)); A.ub = t->st_ub; }
+  if (n > 0 && !is_device_ptr(vartype)) { CUDA_TRY(cudaMemcpyAsync(mat->st_vt, vartype, n, cudaMemcpyDefault, st)); A.vt = mat->st_vt; }
+  if (m > 0 && !is_device_ptr(lhs)) { CUDA_TRY(cudaMemcpyAsync(mat->st_lhs, lhs, 8 * m, cudaMemcpyDefault, st)); A.lhs = mat->st_lhs; }
+  if (m > 0 && !is_device_ptr(rhs)) { CUDA_TRY(cudaMemcpyAsync(mat->st_rhs, rhs, 8 * m, cudaMemcpyDefault, st)); A.rhs = mat->st_rhs; }
+  A.lb_out = hol ? t->out_lb : lb_out;
+  A.ub_out = hou ? t->out_ub : ub_out;
+  A.in_stride = (int64_t)n;
+  A.res = t->h_res;
+  A.count = count;
+  A.sides_ready = 1;
+  team_params(A, p);
+  CUDA_TRY(dp::launch_cluster_teams(A, teams, 1 << k, ctx->num_sms, st));
+  if (hol) CUDA_TRY(cudaMemcpyAsync(lb_out, A.lb_out, bytes, cudaMemcpyDefault, st));
+  if (hou) CUDA_TRY(cudaMemcpyAsync(ub_out, A.ub_out, bytes, cudaMemcpyDefault, st));
+  CUDA_TRY(cudaStreamSynchronize(st));
+  bool any_cap = false;
+  for (int32_t i = 0; i < count; ++i)
+    if (t->h_res[i].w) return t->h_res[i].w;
+  for (int32_t i = 0; i < count; ++i) {
+    const int4 r = t->h_res[i];
+    infeasible[i] = r.x;
+    rounds[i] = r.y;
+    if (status) status[i] = r.z;
+    any_cap |= r.z != 0;
+  }
+  return any_cap ? DP_CAP_HIT : DP_OK;
+}
+
+// Whether a team per node beats the batched kernels.
+bool teams_for_nodes(const dp_ctx *ctx, const dp_matrix *mat, int32_t count) {
+  if (!mat->h_res || ctx->teams_of[0] <= 0) return false;
+  return mat->M.nnz <= kTeamNodeNnz && mat->M.nnz * (int64_t)count <= kTeamNodeWork;
+}
+
 // How a dp_propagate_nodes call runs its rounds: the captured graph (a
 // WHILE loop of the round kernels), the host (one synchronisation per round,
 // so that each stage can be timed with CUDA events), or one persistent
@@ -1108,6 +1403,9 @@ int nodes_call(dp_ctx *ctx, const dp_matrix *cmat, int32_t count, const double *
   const int32_t slab = batch_slab(mat);
   if (slab < 32) return DP_ERR_INVALID_ARG;
   CUDA_TRY(cudaSetDevice(ctx->device));
+  if (mode == kNodesGraph && teams_for_nodes(ctx, mat, count))
+    return nodes_by_teams(ctx, mat, count, lb, ub, vartype, lhs, rhs, p, lb_out, ub_out,
+                          infeasible, rounds, status);
   cudaStream_t st = ctx->stream;
   {
     const int32_t want = count < slab ? (count + 31) / 32 * 32 : slab;

@@ -38,6 +38,7 @@ int64_t live_allocs();
 constexpr int kSliceW = 32;                 // chunks per slice (= warp width)
 constexpr int32_t kLenMask = 0x3FFFFFFF;    // chunk length bits
 constexpr int32_t kExactFlag = 1 << 30;     // row must skip the FP32 screen
+constexpr int32_t kLongSlots = 32;          // slots from which a slice counts as long
 constexpr int kShortRow = 12;               // longest row whose screen values stay in registers
 constexpr int32_t kLayoutEll = 0;           // sliced ELL over row chunks
 constexpr int32_t kLayoutMerge = 1;         // merge-path segments over CSR
@@ -122,6 +123,8 @@ struct DevMatrix {
   int32_t nslices_split;  // slices [0, nslices_split) hold split-row chunks
   int32_t nsplit_rows;
   int32_t round_warps;      // warps per block of the round kernel (4 or 8)
+  int32_t long_split, long_whole;  // slices of kLongSlots slots and more: the first ones of
+                                   // the split slices and of the others
   int32_t short0;           // first slice whose rows all have kShortRow slots at most
   const double *val;        // padded slot-major values
   const int8_t *val8;       // the same values as int8 when all are small
@@ -134,6 +137,10 @@ struct DevMatrix {
   const int32_t *chunk_sidx;// [nslices_split*32] split-row index, -1 = none
   const int32_t *split_row; // [nsplit_rows] row id of each split row
   const int32_t *split_cbeg;// [nsplit_rows+1] range of each split row in split_cidx
+  // column lists for the marking (null in the merge-path layout): the chunk
+  // slots of variable j's nonzeros are col_slot[col_ptr[j] .. col_ptr[j+1])
+  const int32_t *col_ptr;   // [n+1]
+  const int32_t *col_slot;  // [nnz]
   const int32_t *split_cidx;// chunk slots of the split rows' pieces, row by row
                             // (merge path: piece indices, 2t = head of
                             // segment t, 2t+1 = its carry)
@@ -184,6 +191,63 @@ struct DevState {
   uint32_t *dirty;      // [ceil(n/32)] bit j: x_j's next state changed this round
   unsigned *bar;        // [2] grid barrier of the persistent loop: arrivals, generation
   InstState I;          // problem sets only
+};
+
+// ----------------------------------------------------------------- teams --
+//
+// A team is a thread block cluster that runs whole propagations by itself
+// (dp_team.cu).
+
+// One problem of a set as ranges of the union's arrays.
+struct TeamView {
+  int32_t split0, split1;  // slices of split-row chunks
+  int32_t whole0, whole1;  // slices of whole rows
+  int32_t srow0, srow1;    // split rows
+  int32_t var0, var1;      // variables
+  int64_t dword0;          // first word of its dirty bitmap
+  int32_t nlsplit, nlwhole;  // long slices: the first ones of both ranges
+  int32_t id, pad;         // its index among the results
+};
+
+// Per-team words of a running propagation; the pairs are used by even and
+// odd rounds in turn.
+struct TeamFlags {
+  int32_t changed[2];   // a candidate was accepted
+  int32_t infeasible[2];
+  int32_t touched[2];   // a piece of a split row was recomputed
+  int32_t all_next[2];  // too many variables changed to mark their rows one by one
+  int32_t nchanged[2];  // variables committed
+  int32_t err;          // DP_ERR_* found in the inputs
+  int32_t item;         // what the team works on next
+};
+
+struct TeamArgs {
+  DevMatrix M;
+  // state of one propagation, `slots` times (a team owns one); strides in
+  // elements, 0 when there is one team
+  VarRec *rec;
+  longlong2 *keys;
+  uint32_t *dirty;
+  uint32_t *mask;        // [2 * nslices] chunks marked for even and for odd rounds
+  int32_t *touch;
+  Partial *part;
+  RowTot *rowtot;
+  TeamFlags *flags;
+  int64_t s_var, s_dirty, s_mask, s_touch, s_part;
+  double2 *side;         // [chunk slots], shared by all
+  const TeamView *views; // [count] problems of a set, or null: the whole matrix
+  int32_t *next;         // items handed out beyond the first of each team
+  // inputs and outputs: item i's bounds start at i * in_stride
+  const double *lb, *ub, *lhs, *rhs;
+  const uint8_t *vt;
+  double *lb_out, *ub_out;
+  int64_t in_stride;
+  int4 *res;             // [count] {infeasible, rounds, stopped by the cap, error}
+  int32_t count;
+  int32_t sides_ready;   // `side` holds this call's sides
+  int32_t node_sums;     // split rows' sums associated as the batched nodes' kernels do
+  int32_t max_rounds;
+  double eps_int, tau_rel, eps_feas, inf_thr;
 };
 
 // ------------------------------------------------------ batched B&B nodes --

@@ -29,6 +29,16 @@ cudaError_t launch_round_kernels(const DevMatrix &M, const DevState &S,
                                  int use_cond, int num_sms, cudaStream_t st,
                                  cudaEvent_t *ev);
 
+// Teams (dp_team.cu).  launch_columns fills the column lists col_ptr[n+1] and
+// col_slot[nnz] of a sliced-layout matrix (count[n] is scratch).
+// launch_cluster_teams runs A.count items on `teams` clusters of `size` blocks, each with its slot of the state
+// (cluster_teams_resident: how many fit at once; 0 if the size is refused).
+cudaError_t launch_columns(const DevMatrix &M, int32_t *count, int32_t *col_ptr,
+                           int32_t *col_slot, int num_sms, cudaStream_t st);
+int cluster_teams_resident(int size);
+cudaError_t launch_cluster_teams(const TeamArgs &A, int teams, int size, int num_sms,
+                                 cudaStream_t st);
+
 // One launch of the round's memory access pattern without its arithmetic
 // (k_floor; sliced layout only) on `st`.
 cudaError_t launch_access_floor(const DevMatrix &M, const DevState &S, unsigned *sink,
@@ -114,6 +124,13 @@ struct HostLayout {
 int build_layout(int32_t m, int32_t n, int64_t nnz, const int64_t *row_ptr,
                  const int32_t *col_idx, const double *val, int32_t chunk,
                  const double *lhs_hint, const double *rhs_hint, HostLayout &out);
+
+// The layout of several problems' block-diagonal union, problem by problem,
+// and each problem's view of it (largest problem first).
+int build_set_layout(int32_t count, const int32_t *m, const int32_t *n,
+                     const int64_t *const *row_ptr, const int32_t *const *col_idx,
+                     const double *const *val, int32_t chunk, const double *const *lhs,
+                     const double *const *rhs, HostLayout &out, std::vector<TeamView> &views);
 
 // The same for the merge-path layout with `ipt` items per segment
 // (4..4096).

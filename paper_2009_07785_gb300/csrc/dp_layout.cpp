@@ -2,6 +2,7 @@
 // matrix precomputed on the CPU" that Sec. 4.3 of arXiv 2009.07785 excludes
 // from timing): CSR validation, row chunking, length sorting and the
 // slot-major slice image described in dp_internal.h.
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
@@ -198,6 +199,123 @@ int build_layout(int32_t m, int32_t n, int64_t nnz, const int64_t *row_ptr,
         if (small) out.val8[(size_t)(base + (int64_t)k * kSliceW)] = (int8_t)val[ch.begin + k];
       }
     }
+  } catch (const std::bad_alloc &) {
+    return DP_ERR_OOM;
+  }
+  return DP_OK;
+}
+
+// The block-diagonal union of several problems, laid out problem by problem:
+// each problem's slices are those of build_layout on it alone (so a team can
+// take one problem), first the split slices of all problems, then the others.
+int build_set_layout(int32_t count, const int32_t *m, const int32_t *n,
+                     const int64_t *const *row_ptr, const int32_t *const *col_idx,
+                     const double *const *val, int32_t chunk, const double *const *lhs,
+                     const double *const *rhs, HostLayout &out, std::vector<TeamView> &views) {
+  try {
+    std::vector<HostLayout> part((size_t)count);
+    out = HostLayout();
+    bool small = true;
+    int64_t slices = 0, slots = 0;
+    for (int32_t k = 0; k < count; ++k) {
+      HostLayout &P = part[(size_t)k];
+      const int64_t nnz = m[k] > 0 ? row_ptr[k][m[k]] : 0;
+      const int rc = build_layout(m[k], n[k], nnz, row_ptr[k], col_idx[k], val[k], chunk,
+                                  lhs ? lhs[k] : nullptr, rhs ? rhs[k] : nullptr, P);
+      if (rc) return rc;
+      out.m += m[k];
+      out.n += n[k];
+      out.nnz += nnz;
+      out.nslices_split += P.nslices_split;
+      slices += P.nslices;
+      slots += (int64_t)P.val.size();
+      small = small && (nnz == 0 || !P.val8.empty());
+    }
+    // queue entries pack the chunk slot in 30 bits and the element offset in 32
+    if (slices * kSliceW >= (int64_t(1) << 30) || slots >= (int64_t(1) << 32))
+      return DP_ERR_INVALID_ARG;
+    out.nslices = (int32_t)slices;
+    out.val.reserve((size_t)slots);
+    out.col.reserve((size_t)slots);
+    if (small) out.val8.reserve((size_t)slots);
+    views.assign((size_t)count, TeamView());
+    int32_t var = 0, row = 0, srow = 0;
+    int64_t dword = 0;
+    std::vector<int32_t> var0((size_t)count), row0((size_t)count), srow0((size_t)count);
+    for (int32_t k = 0; k < count; ++k) {
+      const HostLayout &P = part[(size_t)k];
+      TeamView &V = views[(size_t)k];
+      V.id = k;
+      V.var0 = var;
+      V.var1 = var + n[k];
+      V.srow0 = srow;
+      V.srow1 = srow + P.nsplit_rows;
+      V.dword0 = dword;
+      var0[(size_t)k] = var;
+      row0[(size_t)k] = row;
+      srow0[(size_t)k] = srow;
+      var += n[k];
+      row += m[k];
+      srow += P.nsplit_rows;
+      dword += ((int64_t)n[k] + 31) / 32;
+    }
+    out.nsplit_rows = srow;
+    // slices [a, b) of problem k, appended
+    auto append = [&](int32_t k, int32_t a, int32_t b) {
+      const HostLayout &P = part[(size_t)k];
+      const int64_t e0 = a < P.nslices ? P.slice_off[(size_t)a] : (int64_t)P.val.size();
+      const int64_t e1 = b < P.nslices ? P.slice_off[(size_t)b] : (int64_t)P.val.size();
+      const int64_t at = (int64_t)out.val.size();
+      for (int32_t q = a; q < b; ++q) {
+        out.slice_off.push_back(at + P.slice_off[(size_t)q] - e0);
+        out.slice_len.push_back(P.slice_len[(size_t)q]);
+        for (int t = 0; t < kSliceW; ++t) {
+          const size_t c = (size_t)q * kSliceW + (size_t)t;
+          out.chunk_row.push_back(P.chunk_row[c] < 0 ? -1 : P.chunk_row[c] + row0[(size_t)k]);
+          out.chunk_len.push_back(P.chunk_len[c]);
+          if (q < P.nslices_split)
+            out.chunk_sidx.push_back(P.chunk_sidx[c] < 0 ? -1
+                                                         : P.chunk_sidx[c] + srow0[(size_t)k]);
+        }
+      }
+      out.val.insert(out.val.end(), P.val.begin() + e0, P.val.begin() + e1);
+      if (small) {
+        if (P.val8.empty()) out.val8.insert(out.val8.end(), (size_t)(e1 - e0), 0);
+        else out.val8.insert(out.val8.end(), P.val8.begin() + e0, P.val8.begin() + e1);
+      }
+      for (int64_t e = e0; e < e1; ++e)
+        out.col.push_back(P.col[(size_t)e] + var0[(size_t)k]);
+    };
+    out.split_cbeg.push_back(0);
+    for (int32_t k = 0; k < count; ++k) {
+      const HostLayout &P = part[(size_t)k];
+      TeamView &V = views[(size_t)k];
+      V.split0 = (int32_t)out.slice_len.size();
+      for (int32_t q = 0; q < P.nslices_split; ++q) V.nlsplit += P.slice_len[(size_t)q] >= kLongSlots;
+      for (int32_t r = 0; r < P.nsplit_rows; ++r) {
+        out.split_row.push_back(P.split_row[(size_t)r] + row0[(size_t)k]);
+        for (int32_t q = P.split_cbeg[(size_t)r]; q < P.split_cbeg[(size_t)r + 1]; ++q)
+          out.split_cidx.push_back(P.split_cidx[(size_t)q] + V.split0 * kSliceW);
+        out.split_cbeg.push_back((int32_t)out.split_cidx.size());
+      }
+      append(k, 0, P.nslices_split);
+      V.split1 = (int32_t)out.slice_len.size();
+    }
+    for (int32_t k = 0; k < count; ++k) {
+      const HostLayout &P = part[(size_t)k];
+      TeamView &V = views[(size_t)k];
+      V.whole0 = (int32_t)out.slice_len.size();
+      for (int32_t q = P.nslices_split; q < P.nslices; ++q)
+        V.nlwhole += P.slice_len[(size_t)q] >= kLongSlots;
+      append(k, P.nslices_split, P.nslices);
+      V.whole1 = (int32_t)out.slice_len.size();
+    }
+    // the teams take the largest problems first
+    std::vector<int64_t> nnz((size_t)count);
+    for (int32_t k = 0; k < count; ++k) nnz[(size_t)k] = m[k] > 0 ? row_ptr[k][m[k]] : 0;
+    std::stable_sort(views.begin(), views.end(), [&](const TeamView &x, const TeamView &y) {
+      return nnz[(size_t)x.id] > nnz[(size_t)y.id];
+    });
   } catch (const std::bad_alloc &) {
     return DP_ERR_OOM;
   }

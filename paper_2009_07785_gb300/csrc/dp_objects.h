@@ -13,6 +13,7 @@ struct dp_ctx {
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   dp::Ctrl *h_ctrl = nullptr;  // pinned mirror of the device control block
+  int teams_of[5] = {0, 0, 0, 0, 0};  // teams of 1, 2, 4, 8, 16 blocks that fit at once
   int live_matrices = 0;
   long long wait_limit = dp::kDefaultWaitLimit;  // grid-barrier wait of the persistent loop
 };
@@ -31,13 +32,35 @@ struct dp_matrix {
   // the round loop
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
+  // one team over the arrays above (dp_team.cu; sliced layout only)
+  dp::TeamFlags *team_flags = nullptr;
+  uint32_t *team_mask = nullptr;   // [2 * nslices]
+  int32_t *team_touch = nullptr;   // [split rows]
+  int4 *h_res = nullptr;           // pinned
   // batched nodes (allocated on the first dp_propagate_nodes call)
   struct BatchWs *batch = nullptr;
+  struct TeamWs *teams = nullptr;  // few nodes of a small matrix: a team each
   const int8_t *val8 = nullptr;  // int8 copy of the values (small integers only)
   // problem sets (dp_matrix_load_set): first row / variable of each problem
   int32_t ninst = 0;
   std::vector<int32_t> row_off, var_off;
   int32_t *h_inst = nullptr;  // pinned [3*ninst]: infeasible, rounds, status
+  dp::TeamView *d_views = nullptr;  // [ninst] the problems, largest first
+  int64_t largest = 0;              // nonzeros of the largest problem
+  int32_t view_slices = 0;          // and its slices
+  int32_t *team_next = nullptr;
+};
+
+// State of `slots` teams (dp_team.cu) that work side by side.
+struct TeamWs {
+  int32_t slots = 0;
+  std::vector<void *> allocs;
+  dp::TeamArgs A{};             // the state's pointers and strides
+  int4 *h_res = nullptr;        // pinned [res_cap]
+  int32_t res_cap = 0;
+  // staging of host inputs / outputs, [stage_cap] bound vectors
+  double *st_lb = nullptr, *st_ub = nullptr, *out_lb = nullptr, *out_ub = nullptr;
+  int64_t stage_cap = 0;
 };
 
 // Workspace of dp_propagate_nodes for up to Bp_cap nodes per launch.

@@ -16,6 +16,18 @@ __device__ __forceinline__ void top2_add(float t, int k, float &t1, float &t2, i
   }
 }
 
+// Adds another part's top-2 (s1 >= s2, slot ks of s1).
+__device__ __forceinline__ void top2_merge(float s1, float s2, int ks, float &t1, float &t2,
+                                           int32_t &k1) {
+  if (s1 > t1) {
+    t2 = fmaxf(t1, s2);
+    t1 = s1;
+    k1 = ks;
+  } else {
+    t2 = fmaxf(t2, s1);
+  }
+}
+
 __device__ __forceinline__ Top2 top2_init() {
   Top2 t;
   t.r1 = t.r2 = t.l1 = t.l2 = -f_inf();
