@@ -381,21 +381,30 @@ int load_layout(dp_ctx *ctx, dp::HostLayout &H, const std::vector<int32_t> *row_
   M.nslices_split = H.nslices_split;
   M.nsplit_rows = H.nsplit_rows;
   M.round_warps = 8;
-  // a single problem's whole rows are sorted by length, longest first
-  M.short0 = H.nslices;
-  while (H.layout == dp::kLayoutEll && !row_off && M.short0 > H.nslices_split &&
-         H.slice_len[(size_t)M.short0 - 1] <= dp::kShortRow)
-    --M.short0;
   M.layout = H.layout;
   M.mp_ipt = H.mp_ipt;
   M.mp_nseg = H.mp_nseg;
   M.mp_nlong = H.mp_nlong;
   M.mp_npiece = (int32_t)H.mp_piece.size();
-  if (H.layout == dp::kLayoutEll) {  // both kinds of slices are sorted, longest first
-    auto is_long = [&](int32_t q) { return H.slice_len[(size_t)q] >= dp::kLongSlots; };
-    while (M.long_split < M.nslices_split && is_long(M.long_split)) ++M.long_split;
-    while (M.nslices_split + M.long_whole < M.nslices && is_long(M.nslices_split + M.long_whole))
-      ++M.long_whole;
+  // the order in which a round takes the slices
+  std::vector<int32_t> order;
+  M.short0 = H.nslices;
+  if (H.layout == dp::kLayoutEll) {
+    auto len = [&](int32_t q) { return H.slice_len[(size_t)q]; };
+    auto is_short = [&](int32_t q) { return q >= H.nslices_split && len(q) <= dp::kShortRow; };
+    for (int32_t q = 0; q < H.nslices; ++q) M.nlong += len(q) >= dp::kLongSlots;
+    if (row_off) {
+      order.resize((size_t)H.nslices);
+      for (int32_t q = 0; q < H.nslices; ++q) order[(size_t)q] = q;
+      std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) {
+        return is_short(x) != is_short(y) ? is_short(y) : len(x) > len(y);
+      });
+      while (M.short0 > 0 && is_short(order[(size_t)M.short0 - 1])) --M.short0;
+    } else {  // both kinds of slices are sorted, longest first
+      while (M.long_split < M.nslices_split && len(M.long_split) >= dp::kLongSlots) ++M.long_split;
+      M.long_whole = M.nlong - M.long_split;
+      while (M.short0 > 0 && is_short(M.short0 - 1)) --M.short0;
+    }
   }
   mat->padded = (int64_t)H.val.size();
 #define TRY(x)                 \
@@ -414,6 +423,7 @@ int load_layout(dp_ctx *ctx, dp::HostLayout &H, const std::vector<int32_t> *row_
   TRY(upload(mat, H.col, &M.col, st));
   TRY(upload(mat, H.slice_off, &M.slice_off, st));
   TRY(upload(mat, H.slice_len, &M.slice_len, st));
+  if (!order.empty()) TRY(upload(mat, order, &M.order, st));
   TRY(upload(mat, H.chunk_row, &M.chunk_row, st));
   TRY(upload(mat, H.chunk_len, &M.chunk_len, st));
   TRY(upload(mat, H.chunk_sidx, &M.chunk_sidx, st));
@@ -672,7 +682,7 @@ int dp_matrix_access_floor(dp_ctx *ctx, const dp_matrix *mat, int32_t reps, floa
   int rc = DP_OK;
   for (int r = 0; r <= reps && rc == DP_OK; ++r) {  // the first launch warms up
     if (cudaEventRecord(e0, st) != cudaSuccess ||
-        dp::launch_access_floor(mat->M, mat->S, sink, st) != cudaSuccess ||
+        dp::launch_access_floor(mat->M, mat->S, sink, ctx->num_sms, st) != cudaSuccess ||
         cudaEventRecord(e1, st) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess) {
       cudaGetLastError();
       rc = DP_ERR_CUDA;

@@ -125,7 +125,11 @@ struct DevMatrix {
   int32_t round_warps;      // warps per block of the round kernel (4 or 8)
   int32_t long_split, long_whole;  // slices of kLongSlots slots and more: the first ones of
                                    // the split slices and of the others
-  int32_t short0;           // first slice whose rows all have kShortRow slots at most
+  const int32_t *order;     // [nslices] a set's slices in the order the round takes them,
+                            // long ones first, whole short rows last (null: nth_slice)
+  int32_t nlong;            // slices of kLongSlots slots and more
+  int32_t short0;           // position in that order from which on all rows are
+                            // whole and have kShortRow nonzeros at most
   const double *val;        // padded slot-major values
   const int8_t *val8;       // the same values as int8 when all are small
                             // integers and compression is on, else null

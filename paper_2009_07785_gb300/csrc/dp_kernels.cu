@@ -398,13 +398,304 @@ __device__ __forceinline__ void short_slice(const DevMatrix &M, const DevState &
     short_rows<1>(M, S, c, elem0, len, row, exact, sd, need_min, inf_flag);
 }
 
+// What a lane knows about its chunk before it reads any nonzero.
+struct ChunkHead {
+  int64_t c;      // chunk slot
+  int32_t len, row;  // 0 and -1 for padding and a stopped problem's rows
+  bool exact;     // the row skips the binary32 screen
+  double2 sd;     // {lhs, rhs}
+  bool need_min, need_max;  // warp-uniform: some lane's row needs that activity
+  int32_t *inf_flag;
+};
+
+// A side's activity is needed only by rows whose side is finite (Step 2 and
+// the candidates of that side); a warp skips the activity no lane needs
+// (warp-uniform: rows are ordered by side pattern when the sides are known
+// at load time).
+template <bool kMulti>
+__device__ __forceinline__ ChunkHead chunk_head(const DevMatrix &M, const DevState &S,
+                                                int slice) {
+  ChunkHead h;
+  h.c = (int64_t)slice * kSliceW + (threadIdx.x & 31);
+  const int32_t lenf = M.chunk_len[h.c];
+  h.len = lenf & kLenMask;
+  h.exact = (lenf & kExactFlag) != 0;
+  h.row = M.chunk_row[h.c];
+  h.inf_flag = &S.ctrl->infeasible;
+  if (kMulti && h.row >= 0) {  // a stopped problem's rows do nothing
+    const int32_t inst = S.I.slot_inst[h.c];
+    if (S.I.done[inst]) {
+      h.row = -1;
+      h.len = 0;
+    } else {
+      h.inf_flag = &S.I.infeasible[inst];
+    }
+  }
+  h.sd = (h.row >= 0) ? S.side[h.c] : make_double2(0.0, 0.0);  // slot order
+  h.need_min = __any_sync(kFull, h.row >= 0 && d_isfinite(h.sd.y));
+  h.need_max = __any_sync(kFull, h.row >= 0 && d_isfinite(h.sd.x));
+  return h;
+}
+
+// A chunk's infinity counts and screen top-2, lane-level; the finite sums
+// are kept apart (round_slice adds them here, team_slice in its chain).
+struct ChunkAcc {
+  int32_t mininf, maxinf;
+  Top2 t;
+};
+
+// One nonzero's contribution apart from the finite sums; returns the
+// bounds those sums use (0 in the place of an infinite one).
+__device__ __forceinline__ void acc_nnz(double av, double L, double U, float WU, float WL, int k,
+                                        bool need_min, bool need_max, ChunkAcc &r, double &bmin,
+                                        double &bmax) {
+  const bool pos = d_pos(av);
+  const float au = absup_fast(av), ad = absdn_fast(av);
+  if (need_min) {
+    bmin = pos ? L : U;
+    const bool inf = d_isinf(bmin);
+    r.mininf += inf;
+    if (inf) r.t.kinf_min = k;
+    bmin = inf ? 0.0 : bmin;
+    top2_add(screen_prod(au, ad, pos ? WU : WL), k, r.t.r1, r.t.r2, r.t.kr);
+  }
+  if (need_max) {
+    bmax = pos ? U : L;
+    const bool inf = d_isinf(bmax);
+    r.maxinf += inf;
+    if (inf) r.t.kinf_max = k;
+    bmax = inf ? 0.0 : bmax;
+    top2_add(screen_prod(au, ad, pos ? WL : WU), k, r.t.l1, r.t.l2, r.t.kl);
+  }
+}
+
+// The coefficient stream: binary64, or the int8 copy (converted when used,
+// so that the prefetched loads stay in flight).
+template <bool kVal8>
+using Raw = typename std::conditional<kVal8, int, double>::type;
+template <bool kVal8>
+__device__ __forceinline__ Raw<kVal8> ld_raw(const DevMatrix &M, int64_t off) {
+  if constexpr (kVal8) return (int)__ldcs(M.val8 + off);
+  else return __ldcs(M.val + off);
+}
+template <bool kVal8>
+__device__ __forceinline__ double coef_of(Raw<kVal8> r) {
+  if constexpr (kVal8) return small_int_to_double(r);
+  else return r;
+}
+
+__device__ __forceinline__ void put_partial(const ChunkHead &h, const ChunkAcc &r, double minfin,
+                                            double maxfin, const DevState &S) {
+  Partial p;
+  p.minfin = minfin;
+  p.maxfin = maxfin;
+  p.mininf = r.mininf;
+  p.maxinf = r.maxinf;
+  p.t = r.t;
+  p.exact = h.exact ? 1 : 0;
+  p.pad = 0;
+  S.part[h.c] = p;
+}
+
+// Step 2 and the screen thresholds of the lane's whole row.
+__device__ __forceinline__ RowView whole_row(const ChunkHead &h, const ChunkAcc &r, double minfin,
+                                             double maxfin, double eps_feas) {
+  RowView rv;
+  rv.minfin = minfin;
+  rv.maxfin = maxfin;
+  rv.mininf = r.mininf;
+  rv.maxinf = r.maxinf;
+  rv.exact = h.exact ? 1 : 0;
+  rv.act = 0;
+  rv.thr_r = rv.thr_l = f_inf();
+  rv.lhs = h.sd.x;
+  rv.rhs = h.sd.y;
+  if (h.row >= 0) row_sides(rv, r.t.r1, r.t.l1, eps_feas, h.inf_flag);
+  return rv;
+}
+
+// ---- long slices: one slice per block ----
+//
+// A lane of round_slice spends about 0.17 us per slot on dependent
+// instructions alone (plus the latency of each group's gathers), so a slice
+// of 256 slots takes 70-110 us however empty the GPU is, and on a matrix
+// with any long row that is what the round waits for (2M nonzeros with rows of
+// 20,000 to 50,000: 70 -> 40 us per round; 6M with rows of up to 100,000: 99 ->
+// 61).  A block costs 1.5 times the warp-time per slice, so it pays while the
+// blocks' slices are few (30M nonzeros, 15 long slices per SM: 210 -> 340).  Here the block's
+// warps take U consecutive slots each, so that loads, gathers and the screen
+// run side by side; the bounds go through shared memory to one warp per side
+// that adds them slot by slot.  The finite sums thus stay one FMA chain per
+// row in CSR order, the same bits as round_slice, and the chain (about 64
+// clocks per slot: the binary64 pipe) is all that remains serial.
+constexpr int kTeamU = 2;            // slots per warp and step
+constexpr int kTeamBlocksPerSM = 4;  // long slices per SM up to which a block takes each
+
+struct TeamPart {  // one warp's share of a chunk
+  ChunkAcc r;
+};
+
+template <int kWarps>
+struct TeamBuf {
+  static constexpr int kStep = kWarps * kTeamU;
+  union {
+    double b[2][2][kStep][kSliceW];      // [side][buffer][slot][lane] bounds of a step
+    TeamPart part[kWarps][kSliceW];
+  };
+  double fin[2][kSliceW];
+  RowView rv[kSliceW];
+  int32_t len[kSliceW];  // slots to re-read of each chunk
+};
+
+template <bool kMulti, int kWarps, bool kVal8>
+__device__ __forceinline__ void team_slice(const DevMatrix &M, const DevState &S, int slice,
+                                           TeamBuf<kWarps> &sb) {
+  constexpr int U = kTeamU, kStep = TeamBuf<kWarps>::kStep;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const ChunkHead h = chunk_head<kMulti>(M, S, slice);
+  const int32_t len = h.len;
+  const int maxlen = __reduce_max_sync(kFull, len);  // the same in every warp
+  const int64_t vo = M.slice_off[slice] + lane;
+  const int32_t *cp = M.col + vo;
+  const bool need_min = h.need_min, need_max = h.need_max;
+  // the warps that add up the sides: on different binary64 pipes, and not
+  // the same ones in every block
+  const int wmin = blockIdx.x % kWarps, wmax = (blockIdx.x + 1) % kWarps;
+  double fin = 0.0;
+  ChunkAcc r;
+  r.mininf = r.maxinf = 0;
+  r.t = top2_init();
+  Raw<kVal8> an[U];
+  int32_t jn[U];
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      an[u] = (Raw<kVal8>)1;
+      jn[u] = 0;
+      if (k0 + u < len) {
+        if constexpr (kVal8) an[u] = (int)__ldg(M.val8 + vo + (int64_t)(k0 + u) * kSliceW);
+        else an[u] = __ldg(M.val + vo + (int64_t)(k0 + u) * kSliceW);
+        jn[u] = __ldg(cp + (int64_t)(k0 + u) * kSliceW);
+      }
+    }
+  };
+  // adds the staged step that began at slot s0 (its coefficients are in L1)
+  auto chain = [&](int s0, int side) {
+    const double(*bb)[kSliceW] = sb.b[side][(s0 / kStep) & 1];
+    for (int q = 0; q < kStep; q += 4) {
+      Raw<kVal8> a[4];
+      double b[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        a[u] = (Raw<kVal8>)1;
+        b[u] = 0.0;
+        if (s0 + q + u < len) {
+          if constexpr (kVal8) a[u] = (int)__ldg(M.val8 + vo + (int64_t)(s0 + q + u) * kSliceW);
+          else a[u] = __ldg(M.val + vo + (int64_t)(s0 + q + u) * kSliceW);
+          b[u] = bb[q + u][lane];
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (s0 + q + u < len) fin = fma(coef_of<kVal8>(a[u]), b[u], fin);
+    }
+  };
+  fetch(warp * U);
+  for (int s = 0; s < maxlen; s += kStep) {
+    const int k = s + warp * U;
+    Raw<kVal8> a[U];
+    double L[U], Ub[U];
+    float WU[U], WL[U];
+    uint32_t fl[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      a[u] = an[u];
+      L[u] = Ub[u] = 0.0;
+      WU[u] = WL[u] = 0.0f;
+      if (k + u < len) ld_rec(S.rec + jn[u], L[u], Ub[u], WU[u], WL[u], fl[u]);
+    }
+    fetch(k + kStep);
+    if (s > 0 && need_min && warp == wmin) chain(s - kStep, 0);
+    if (s > 0 && need_max && warp == wmax) chain(s - kStep, 1);
+    const int buf = (s / kStep) & 1;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (k + u < len) {
+        double bmin, bmax;
+        acc_nnz(coef_of<kVal8>(a[u]), L[u], Ub[u], WU[u], WL[u], k + u, need_min, need_max, r,
+                bmin, bmax);
+        if (need_min) sb.b[0][buf][warp * U + u][lane] = bmin;
+        if (need_max) sb.b[1][buf][warp * U + u][lane] = bmax;
+      }
+    }
+    __syncthreads();  // the step is staged, and the step before it is added
+  }
+  if (maxlen > 0) {
+    const int last = (maxlen - 1) / kStep * kStep;
+    if (need_min && warp == wmin) chain(last, 0);
+    if (need_max && warp == wmax) chain(last, 1);
+    __syncthreads();  // the staging is free for the warps' parts
+  }
+  sb.part[warp][lane].r = r;
+  if (warp == wmin) sb.fin[0][lane] = need_min ? fin : 0.0;
+  if (kWarps > 1 && warp == wmax) sb.fin[1][lane] = need_max ? fin : 0.0;
+  __syncthreads();
+  if (warp == 0) {
+#pragma unroll 1
+    for (int w = 1; w < kWarps; ++w) {
+      const ChunkAcc q = sb.part[w][lane].r;
+      if (q.mininf > 0) r.t.kinf_min = q.t.kinf_min;
+      if (q.maxinf > 0) r.t.kinf_max = q.t.kinf_max;
+      r.mininf += q.mininf;
+      r.maxinf += q.maxinf;
+      top2_merge(q.t.r1, q.t.r2, q.t.kr, r.t.r1, r.t.r2, r.t.kr);
+      top2_merge(q.t.l1, q.t.l2, q.t.kl, r.t.l1, r.t.l2, r.t.kl);
+    }
+    if (h.exact) r.t.r1 = r.t.r2 = r.t.l1 = r.t.l2 = f_inf();
+    const double minfin = sb.fin[0][lane], maxfin = sb.fin[1][lane];
+    if (slice < M.nslices_split) {
+      if (h.row >= 0) put_partial(h, r, minfin, maxfin, S);
+    } else {
+      const RowView rv = whole_row(h, r, minfin, maxfin, S.ctrl->eps_feas);
+      const bool full =
+          enqueue_named<kSliceW>(rv, r.t, r.mininf, r.maxinf, h.c, vo, S);
+      sb.rv[lane] = rv;
+      sb.len[lane] = full ? len : 0;
+    }
+  }
+  if (slice < M.nslices_split) return;  // block-uniform
+  __syncthreads();
+  // the re-read of rows with several survivors, shared by the warps
+  const int32_t rlen = sb.len[lane];
+  if (__ballot_sync(kFull, rlen > 0) == 0u) return;
+  const RowView rv = sb.rv[lane];
+  enqueue_reread<kSliceW, false>(rv, rlen, warp * 4, kWarps * 4, h.c, vo, M, M.col, S);
+}
+
+// The q-th slice of a round, the long ones first.
+__device__ __forceinline__ int nth_slice(const DevMatrix &M, int q) {
+  if (M.order) return M.order[q];
+  const int nlong = M.long_split + M.long_whole;
+  if (q < nlong) return q < M.long_split ? q : M.nslices_split + (q - M.long_split);
+  q -= nlong;
+  const int rest = M.nslices_split - M.long_split;  // split slices that are not long
+  return q < rest ? M.long_split + q : M.nslices_split + M.long_whole + (q - rest);
+}
+
+// The first `teams` slices by a block each, the others by a warp each.
 template <bool kMulti, int kRoundWarps, bool kVal8>
 __global__ void __launch_bounds__(kRoundWarps * 32, kRoundWarpsPerSM / kRoundWarps)
-k_round(DevMatrix M, DevState S) {
+k_round(DevMatrix M, DevState S, int teams) {
+  __shared__ TeamBuf<kRoundWarps> sb;
   if (S.ctrl->err) return;
-  const int slice = blockIdx.x * kRoundWarps + (threadIdx.x >> 5);
-  if (slice >= M.nslices) return;  // warp-uniform
-  if (!kVal8 && slice >= M.short0) short_slice<kMulti>(M, S, slice);
+  if ((int)blockIdx.x < teams) {
+    team_slice<kMulti, kRoundWarps, kVal8>(M, S, nth_slice(M, blockIdx.x), sb);
+    return;
+  }
+  const int q = teams + ((int)blockIdx.x - teams) * kRoundWarps + (threadIdx.x >> 5);
+  if (q >= M.nslices) return;  // warp-uniform
+  const int slice = nth_slice(M, q);
+  if (!kVal8 && q >= M.short0) short_slice<kMulti>(M, S, slice);
   else round_slice<kMulti, kVal8>(M, S, slice);
 }
 
@@ -418,15 +709,20 @@ k_round(DevMatrix M, DevState S) {
 // of propagation).
 template <int kRoundWarps>
 __global__ void __launch_bounds__(kRoundWarps * 32, kRoundWarpsPerSM / kRoundWarps)
-k_floor(DevMatrix M, DevState S, unsigned *sink) {
-  const int slice = blockIdx.x * kRoundWarps + (threadIdx.x >> 5);
-  if (slice >= M.nslices) return;
+k_floor(DevMatrix M, DevState S, int teams, unsigned *sink) {
+  const int warp = threadIdx.x >> 5;
+  const bool team = (int)blockIdx.x < teams;  // its warps share the slice's slots
+  const int q = team ? (int)blockIdx.x
+                     : teams + ((int)blockIdx.x - teams) * kRoundWarps + warp;
+  if (q >= M.nslices) return;
+  const int slice = nth_slice(M, q);
+  const int kbeg = team ? warp * kGroup : 0, kstep = team ? kRoundWarps * kGroup : kGroup;
   const int lane = threadIdx.x & 31;
   const int64_t c = (int64_t)slice * kSliceW + lane;
   const int32_t len = M.chunk_len[c] & kLenMask;
   const int64_t vo = M.slice_off[slice] + lane;
   unsigned acc = 0u;
-  for (int k = 0; k < len; k += kGroup) {
+  for (int k = kbeg; k < len; k += kstep) {
     double a[kGroup];
     int32_t j[kGroup];
 #pragma unroll
@@ -453,14 +749,20 @@ k_floor(DevMatrix M, DevState S, unsigned *sink) {
   if (acc == 0x9E3779B9u) *sink = acc;  // practically never: keeps the loads
 }
 
+// Slices that a block takes each: the long ones, when they are few.
+static int team_blocks(const DevMatrix &M, int num_sms) {
+  return M.nlong <= kTeamBlocksPerSM * num_sms ? M.nlong : 0;
+}
+
 cudaError_t launch_access_floor(const DevMatrix &M, const DevState &S, unsigned *sink,
-                                cudaStream_t st) {
+                                int num_sms, cudaStream_t st) {
   if (M.layout != kLayoutEll) return cudaErrorInvalidValue;
   const int w = M.round_warps == 4 ? 4 : 8;
-  int nb = (M.nslices + w - 1) / w;
+  const int teams = team_blocks(M, num_sms);
+  int nb = teams + (M.nslices - teams + w - 1) / w;
   if (nb < 1) nb = 1;
-  if (w == 4) k_floor<4><<<nb, 4 * 32, 0, st>>>(M, S, sink);
-  else k_floor<8><<<nb, 8 * 32, 0, st>>>(M, S, sink);
+  if (w == 4) k_floor<4><<<nb, 4 * 32, 0, st>>>(M, S, teams, sink);
+  else k_floor<8><<<nb, 8 * 32, 0, st>>>(M, S, teams, sink);
   return cudaGetLastError();
 }
 
@@ -602,53 +904,85 @@ k_combine(DevMatrix M, DevState S) {
 
 // --------------------------------------------------------- k_cand_split --
 
+// The state of the active split rows' chunks of one slice: the row's sums
+// and thresholds, the chunk's top-2 (lane-level).
+struct SplitChunk {
+  RowView rv;
+  Top2 t;
+  int32_t len, mininf, maxinf;
+};
+
+__device__ __forceinline__ SplitChunk split_chunk(const DevMatrix &M, const DevState &S,
+                                                  int64_t c) {
+  SplitChunk x;
+  const int32_t sidx = M.chunk_sidx[c];
+  x.rv.act = 0;
+  x.rv.exact = 0;
+  x.rv.mininf = x.rv.maxinf = 0;
+  x.rv.minfin = x.rv.maxfin = x.rv.lhs = x.rv.rhs = 0.0;
+  x.rv.thr_r = x.rv.thr_l = f_inf();
+  x.t = top2_init();
+  x.len = x.mininf = x.maxinf = 0;
+  if (sidx >= 0) {
+    const RowTot rt = S.rowtot[sidx];
+    if (rt.active) {
+      const Partial p = S.part[c];
+      const int32_t lenf = M.chunk_len[c];
+      x.len = lenf & kLenMask;
+      x.rv.minfin = rt.minfin;
+      x.rv.maxfin = rt.maxfin;
+      x.rv.mininf = rt.mininf;
+      x.rv.maxinf = rt.maxinf;
+      x.rv.thr_r = rt.thr_r;
+      x.rv.thr_l = rt.thr_l;
+      x.rv.lhs = S.lhs[rt.row];
+      x.rv.rhs = S.rhs[rt.row];
+      x.rv.exact = (lenf & kExactFlag) ? 1 : 0;
+      x.rv.act = 1;
+      x.t = p.t;
+      x.mininf = p.mininf;
+      x.maxinf = p.maxinf;
+    }
+  }
+  return x;
+}
+
 // Candidates of the active split rows' chunks of one slice (warp-level).
 template <bool kCo = false>
 __device__ __forceinline__ void cand_split_slice(const DevMatrix &M, const DevState &S,
                                                  int slice) {
   const int lane = threadIdx.x & 31;
   const int64_t c = (int64_t)slice * kSliceW + lane;
-  const int32_t sidx = M.chunk_sidx[c];
-  RowView rv;
-  rv.act = 0;
-  rv.exact = 0;
-  rv.mininf = rv.maxinf = 0;
-  rv.minfin = rv.maxfin = rv.lhs = rv.rhs = 0.0;
-  rv.thr_r = rv.thr_l = f_inf();
-  Top2 t = top2_init();
-  int32_t len = 0, cmin = 0, cmax = 0;
-  if (sidx >= 0) {
-    const RowTot rt = S.rowtot[sidx];
-    if (rt.active) {
-      const Partial p = S.part[c];
-      const int32_t lenf = M.chunk_len[c];
-      len = lenf & kLenMask;
-      rv.minfin = rt.minfin;
-      rv.maxfin = rt.maxfin;
-      rv.mininf = rt.mininf;
-      rv.maxinf = rt.maxinf;
-      rv.thr_r = rt.thr_r;
-      rv.thr_l = rt.thr_l;
-      rv.lhs = S.lhs[rt.row];
-      rv.rhs = S.rhs[rt.row];
-      rv.exact = (lenf & kExactFlag) ? 1 : 0;
-      rv.act = 1;
-      t = p.t;
-      cmin = p.mininf;
-      cmax = p.maxinf;
-    }
-  }
-  const int64_t sbase = M.slice_off[slice];
-  warp_enqueue<kSliceW, kCo>(rv, t, cmin, cmax, len, c, sbase + lane, M, M.col, S);
+  const SplitChunk x = split_chunk(M, S, c);
+  warp_enqueue<kSliceW, kCo>(x.rv, x.t, x.mininf, x.maxinf, x.len, c, M.slice_off[slice] + lane,
+                             M, M.col, S);
 }
 
+// A block per long slice (its warps share the re-read, which one lane's walk
+// made the longest part of early rounds: 30M nonzeros 42 -> 15 us per round), a
+// warp per other one.
 template <int kRoundWarps>
 __global__ void __launch_bounds__(kRoundWarps * 32)
 k_cand_split(DevMatrix M, DevState S) {
   if (S.ctrl->err) return;
-  const int slice = blockIdx.x * kRoundWarps + (threadIdx.x >> 5);
-  if (slice >= M.nslices_split) return;  // warp-uniform
-  cand_split_slice(M, S, slice);
+  __shared__ int32_t s_len[kSliceW];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (blockIdx.x >= M.long_split) {
+    const int slice = M.long_split + ((int)blockIdx.x - M.long_split) * kRoundWarps + warp;
+    if (slice < M.nslices_split) cand_split_slice(M, S, slice);  // warp-uniform
+    return;
+  }
+  const int slice = blockIdx.x;
+  const int64_t c = (int64_t)slice * kSliceW + lane, vo = M.slice_off[slice] + lane;
+  const SplitChunk x = split_chunk(M, S, c);  // the same in every warp
+  if (__ballot_sync(kFull, x.rv.act != 0) == 0u) return;
+  if (warp == 0)
+    s_len[lane] =
+        enqueue_named<kSliceW>(x.rv, x.t, x.mininf, x.maxinf, c, vo, S) ? x.len : 0;
+  __syncthreads();
+  const int32_t rlen = s_len[lane];
+  if (__ballot_sync(kFull, rlen > 0) == 0u) return;
+  enqueue_reread<kSliceW, false>(x.rv, rlen, warp * 4, kRoundWarps * 4, c, vo, M, M.col, S);
 }
 
 // ------------------------------------------------------------- k_finish --
@@ -994,16 +1328,17 @@ cudaError_t launch_epilogue(const DevState &S, int32_t n, double *lb_out, double
 // The sliced-ELL part of a round: activities, split rows, Step 2 and the
 // screen (events ev[0..5] as in launch_round_kernels).
 template <bool kMulti, int kRoundWarps>
-cudaError_t launch_ell_front(const DevMatrix &M, const DevState &S, cudaStream_t st,
-                             cudaEvent_t *ev) {
+cudaError_t launch_ell_front(const DevMatrix &M, const DevState &S, int num_sms,
+                             cudaStream_t st, cudaEvent_t *ev) {
   cudaError_t e;
-  int nb = (M.nslices + kRoundWarps - 1) / kRoundWarps;
+  const int teams = team_blocks(M, num_sms);
+  int nb = teams + (M.nslices - teams + kRoundWarps - 1) / kRoundWarps;
   if (nb < 1) nb = 1;
   if (ev) cudaEventRecord(ev[0], st);
   if (M.val8)
-    k_round<kMulti, kRoundWarps, true><<<nb, kRoundWarps * 32, 0, st>>>(M, S);
+    k_round<kMulti, kRoundWarps, true><<<nb, kRoundWarps * 32, 0, st>>>(M, S, teams);
   else
-    k_round<kMulti, kRoundWarps, false><<<nb, kRoundWarps * 32, 0, st>>>(M, S);
+    k_round<kMulti, kRoundWarps, false><<<nb, kRoundWarps * 32, 0, st>>>(M, S, teams);
   if (ev) cudaEventRecord(ev[1], st);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (M.nsplit_rows > 0) {
@@ -1012,7 +1347,7 @@ cudaError_t launch_ell_front(const DevMatrix &M, const DevState &S, cudaStream_t
     k_combine<kMulti><<<nbc, kCombineWarps * 32, 0, st>>>(M, S);
     if (ev) cudaEventRecord(ev[3], st);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    int nbs = (M.nslices_split + kRoundWarps - 1) / kRoundWarps;
+    const int nbs = M.long_split + (M.nslices_split - M.long_split + kRoundWarps - 1) / kRoundWarps;
     if (ev) cudaEventRecord(ev[4], st);
     k_cand_split<kRoundWarps><<<nbs, kRoundWarps * 32, 0, st>>>(M, S);
     if (ev) cudaEventRecord(ev[5], st);
@@ -1026,7 +1361,7 @@ cudaError_t launch_round_t(const DevMatrix &M, const DevState &S, const uint8_t 
                            cudaGraphConditionalHandle handle, int use_cond, int num_sms,
                            cudaStream_t st, cudaEvent_t *ev) {
   cudaError_t e = M.layout == kLayoutMerge ? launch_merge_front(M, S, num_sms, st, ev)
-                                           : launch_ell_front<kMulti, kRoundWarps>(M, S, st, ev);
+                                           : launch_ell_front<kMulti, kRoundWarps>(M, S, num_sms, st, ev);
   if (e != cudaSuccess) return e;
   // the queue kernel's grid: the blocks that are resident at once (a
   // larger grid-stride grid would run its last blocks as a second wave)

@@ -42,7 +42,7 @@ cudaError_t launch_cluster_teams(const TeamArgs &A, int teams, int size, int num
 // One launch of the round's memory access pattern without its arithmetic
 // (k_floor; sliced layout only) on `st`.
 cudaError_t launch_access_floor(const DevMatrix &M, const DevState &S, unsigned *sink,
-                                cudaStream_t st);
+                                int num_sms, cudaStream_t st);
 
 // The whole round loop as one cooperative (persistent) launch on `st`
 // (single problems only).

@@ -177,51 +177,51 @@ __device__ __forceinline__ int warp_reserve(int c, int32_t *counter) {
   return __shfl_sync(kFull, base, 0) + before;
 }
 
-// Queues nonzeros of the lanes' chunks whose candidates survive the screen.
-// Entries go to a global queue (warp-aggregated slots) and are evaluated by
-// k_cand_queue, one per thread, so the binary64 candidate formulas run
-// lane-dense across the whole GPU however few survivors a warp has.  When
-// the second-largest screen value of a side is below the threshold, only the
-// chunk's largest can survive and it is queued directly (no re-read);
-// otherwise the lane re-reads its chunk (values and columns from L2, records
-// through the same gather), four slots at a time.  Element k of a lane's
-// chunk sits at elem0 + k * kStride of val/col (slot-major slices: the
-// lane's slot in the slice, stride 32; CSR rows: the row's offset, stride
-// 1).  All 32 lanes must call this (warp collectives).  Returns whether the
-// lane's chunk needed the full re-read (done here for its first mylen
-// slots).  kCo: records are loaded through L2 (the persistent loop, which
-// rewrites them between its phases).
-template <int kStride, bool kCo = false>
-__device__ __forceinline__ bool warp_enqueue(const RowView &mine, const Top2 &t, int chunk_mininf,
-                                             int chunk_maxinf, int32_t mylen, int64_t chunk_slot,
-                                             int64_t elem0, const DevMatrix &M,
-                                             const int32_t *col, const DevState &S) {
+// Queueing of the nonzeros of the lanes' chunks whose candidates survive
+// the screen.  Entries go to a global queue (warp-aggregated slots) and are
+// evaluated by k_cand_queue, one per thread, so the binary64 candidate
+// formulas run lane-dense across the whole GPU however few survivors a warp
+// has.  When the second-largest screen value of a side is below the
+// threshold, only the chunk's largest can survive and it is queued directly
+// (enqueue_named, no re-read); otherwise the chunk is re-read
+// (enqueue_reread: values and columns from L2, records through the same
+// gather), four slots at a time.  Element k of a lane's chunk sits at
+// elem0 + k * kStride of val/col (slot-major slices: the lane's slot in the
+// slice, stride 32; CSR rows: the row's offset, stride 1).
+
+__device__ __forceinline__ CandEntry cand_entry(int64_t elem, int64_t chunk_slot,
+                                                unsigned sides) {
+  CandEntry e;
+  e.off = (uint32_t)elem;
+  e.cs = ((uint32_t)chunk_slot << 2) | sides;
+  return e;
+}
+
+__device__ __forceinline__ void put_rowsum(const RowView &mine, int64_t chunk_slot,
+                                           const DevState &S) {
+  RowSum rs;
+  rs.minfin = mine.minfin;
+  rs.maxfin = mine.maxfin;
+  rs.mininf = mine.mininf;
+  rs.maxinf = mine.maxinf;
+  S.rowsum[chunk_slot] = rs;
+}
+
+// Queues the survivors that can be named without re-reading the chunk and
+// writes the row's sums for every lane that has, or may have, an entry.
+// Returns whether the lane's chunk needs the re-read.  All 32 lanes call.
+template <int kStride>
+__device__ __forceinline__ bool enqueue_named(const RowView &mine, const Top2 &t,
+                                              int chunk_mininf, int chunk_maxinf,
+                                              int64_t chunk_slot, int64_t elem0,
+                                              const DevState &S) {
   const bool act = mine.act != 0;
   if (__ballot_sync(kFull, act) == 0u) return false;
-
-  bool wrote_sums = false;
-  auto sums = [&]() {  // the row's sums, once, before its first queued entry
-    if (wrote_sums) return;
-    RowSum rs;
-    rs.minfin = mine.minfin;
-    rs.maxfin = mine.maxfin;
-    rs.mininf = mine.mininf;
-    rs.maxinf = mine.maxinf;
-    S.rowsum[chunk_slot] = rs;
-    wrote_sums = true;
-  };
-  auto entry = [&](int k, unsigned sides) {
-    CandEntry e;
-    e.off = (uint32_t)(elem0 + (int64_t)k * kStride);
-    e.cs = ((uint32_t)chunk_slot << 2) | sides;
-    return e;
-  };
-
-  // Survivors can be named without re-reading the chunk unless a side has
-  // two screen values above its threshold (or the row skips the screen).
-  // With exactly one infinite contribution to a side's activity, only that
-  // nonzero gets a finite residual on that side (Sec. 3.4); its slot was
-  // recorded by the activity pass.
+  // Survivors can be named unless a side has two screen values above its
+  // threshold (or the row skips the screen).  With exactly one infinite
+  // contribution to a side's activity, only that nonzero gets a finite
+  // residual on that side (Sec. 3.4); its slot was recorded by the activity
+  // pass.
   const bool full = act && (mine.exact || (mine.mininf == 0 && t.r2 > mine.thr_r) ||
                             (mine.maxinf == 0 && t.l2 > mine.thr_l));
   bool h1 = false, h2 = false;
@@ -234,20 +234,25 @@ __device__ __forceinline__ bool warp_enqueue(const RowView &mine, const Top2 &t,
     if (fl && mine.maxinf == 1 && chunk_maxinf > 0) { h2 = true; k2 = t.kinf_max; }
   }
   const bool merge = h1 && h2 && k1 == k2;
-  {
-    const bool q2 = h2 && !merge;
-    int pos = warp_reserve((h1 ? 1 : 0) + (q2 ? 1 : 0), &S.ctrl->qcount);
-    if (h1 || q2) sums();
-    if (h1) S.queue[pos++] = entry(k1, merge ? 3u : 1u);
-    if (q2) S.queue[pos] = entry(k2, 2u);
-  }
+  const bool q2 = h2 && !merge;
+  int pos = warp_reserve((h1 ? 1 : 0) + (q2 ? 1 : 0), &S.ctrl->qcount);
+  if (h1 || q2 || full) put_rowsum(mine, chunk_slot, S);
+  if (h1) S.queue[pos++] = cand_entry(elem0 + (int64_t)k1 * kStride, chunk_slot, merge ? 3u : 1u);
+  if (q2) S.queue[pos] = cand_entry(elem0 + (int64_t)k2 * kStride, chunk_slot, 2u);
+  return full;
+}
 
-  // full re-read of the chunk, four slots at a time
-  const int len = full ? mylen : 0;
-  int maxlen = len;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) maxlen = max(maxlen, __shfl_xor_sync(kFull, maxlen, o));
-  const int64_t vo = elem0;
+// Re-reads the lanes' chunks (len slots each, 0 for a lane without one) and
+// queues every nonzero that survives the screen: four slots from `kbeg`,
+// then every `kstep` slots further on (several warps can share the slots of
+// a slice).  kCo: records are loaded through L2 (the persistent loop, which
+// rewrites them between its phases).  All 32 lanes call.
+template <int kStride, bool kCo>
+__device__ __forceinline__ void enqueue_reread(const RowView &mine, int32_t len, int kbeg,
+                                               int kstep, int64_t chunk_slot, int64_t elem0,
+                                               const DevMatrix &M, const int32_t *col,
+                                               const DevState &S) {
+  const int maxlen = __reduce_max_sync(kFull, len);
   const int32_t *cp = col + elem0;
   // software-pipelined: the next group's values and columns are fetched
   // while this group's records are gathered
@@ -259,13 +264,13 @@ __device__ __forceinline__ bool warp_enqueue(const RowView &mine, const Top2 &t,
       an[u] = 1.0;
       jn[u] = 0;
       if (k0 + u < len) {
-        an[u] = ld_coef(M, vo + (int64_t)(k0 + u) * kStride);
+        an[u] = ld_coef(M, elem0 + (int64_t)(k0 + u) * kStride);
         jn[u] = cp[(int64_t)(k0 + u) * kStride];
       }
     }
   };
-  if (maxlen > 0) fetch(0);
-  for (int k = 0; k < maxlen; k += 4) {
+  if (kbeg < maxlen) fetch(kbeg);
+  for (int k = kbeg; k < maxlen; k += kstep) {
     double a[4], L[4], U[4];
     float WU[4], WL[4];
     uint32_t fl[4];
@@ -276,7 +281,7 @@ __device__ __forceinline__ bool warp_enqueue(const RowView &mine, const Top2 &t,
       WU[u] = WL[u] = 0.0f;
       if (k + u < len) ld_rec_t<kCo>(S.rec + jn[u], L[u], U[u], WU[u], WL[u], fl[u]);
     }
-    if (k + 4 < maxlen) fetch(k + 4);
+    if (k + kstep < maxlen) fetch(k + kstep);
     unsigned sd[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u)
@@ -286,11 +291,24 @@ __device__ __forceinline__ bool warp_enqueue(const RowView &mine, const Top2 &t,
 #pragma unroll
     for (int u = 0; u < 4; ++u) c += sd[u] != 0u;
     int pos = warp_reserve(c, &S.ctrl->qcount);
-    if (c > 0) sums();
 #pragma unroll
     for (int u = 0; u < 4; ++u)
-      if (sd[u] != 0u) S.queue[pos++] = entry(k + u, sd[u]);
+      if (sd[u] != 0u)
+        S.queue[pos++] = cand_entry(elem0 + (int64_t)(k + u) * kStride, chunk_slot, sd[u]);
   }
+}
+
+// Both, by one warp.  Returns whether the lane's chunk needed the re-read
+// (done here for its first mylen slots).
+template <int kStride, bool kCo = false>
+__device__ __forceinline__ bool warp_enqueue(const RowView &mine, const Top2 &t, int chunk_mininf,
+                                             int chunk_maxinf, int32_t mylen, int64_t chunk_slot,
+                                             int64_t elem0, const DevMatrix &M,
+                                             const int32_t *col, const DevState &S) {
+  const bool full =
+      enqueue_named<kStride>(mine, t, chunk_mininf, chunk_maxinf, chunk_slot, elem0, S);
+  if (__ballot_sync(kFull, full) == 0u) return false;
+  enqueue_reread<kStride, kCo>(mine, full ? mylen : 0, 0, 4, chunk_slot, elem0, M, col, S);
   return full;
 }
 
