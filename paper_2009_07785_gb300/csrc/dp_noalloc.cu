@@ -351,25 +351,27 @@ __device__ __forceinline__ void na_row_block(const NaArgs &A, NaRow r, int64_t b
   }
 }
 
-// One round, kNaThreads rows per block: short rows by a lane each, longer
-// ones by a warp, the longest by the block.  What bounds a round is the
+// One round, `per` rows (32..kNaThreads, a multiple of 32) per block: short
+// rows by a lane each, longer ones by a warp, the longest by the block.  Few
+// rows are spread over as many blocks as there are, since the lanes' binary64
+// work shares one pipe per scheduler.  What bounds a round is the
 // latency of its longest row: one lane's walk takes about 1 us per nonzero
 // (two dependent loads and the binary64 chain), so a row of 12,000 nonzeros
 // took 12 ms per round where the block takes about 30 us.  A row of up to
 // kNaWarpRow nonzeros is one FMA chain in CSR order whichever way it goes.
 __global__ void __launch_bounds__(kNaThreads)
-k_na_round(int32_t m, const int64_t *row_ptr, const double *lhs_in, const double *rhs_in,
-           NaArgs A) {
+k_na_round(int32_t m, int per, const int64_t *row_ptr, const double *lhs_in,
+           const double *rhs_in, NaArgs A) {
   __shared__ int s_long[kNaThreads];
   __shared__ int s_count;
   if (threadIdx.x == 0) s_count = 0;
   __syncthreads();
-  const int64_t i = blockIdx.x * (int64_t)kNaThreads + threadIdx.x;
+  const int64_t i = blockIdx.x * (int64_t)per + threadIdx.x;
   NaRow r;
   r.minfin = r.maxfin = r.lhs = r.rhs = 0.0;
   r.mininf = r.maxinf = 0;
   int64_t b = 0, e = 0;
-  if (i < m) {
+  if (i < m && (int)threadIdx.x < per) {
     r.lhs = side_norm(lhs_in[i], A.thr);
     r.rhs = side_norm(rhs_in[i], A.thr);
     b = row_ptr[i];
@@ -391,7 +393,7 @@ k_na_round(int32_t m, const int64_t *row_ptr, const double *lhs_in, const double
   __syncthreads();
   const int nlong = s_count;
   for (int q = 0; q < nlong; ++q) {  // block-uniform
-    const int64_t row = blockIdx.x * (int64_t)kNaThreads + s_long[q];
+    const int64_t row = blockIdx.x * (int64_t)per + s_long[q];
     NaRow x;
     x.minfin = x.maxfin = 0.0;
     x.mininf = x.maxinf = 0;
@@ -538,13 +540,15 @@ extern "C" int dp_propagate_noalloc(int device, void *cuda_stream, int32_t m, in
   A.tau = p.tau_rel;
   A.eps_feas = p.eps_feas;
   A.thr = p.inf_threshold;
+  int per = 32;  // rows per block: about 600 blocks and more, four per SM
+  while (per < kNaThreads && m > 600 * per) per *= 2;
   int32_t r = 0;
   bool changed = false;
   for (; r < p.max_rounds;) {
     if (cudaMemsetAsync(ctrl, 0, sizeof(NoallocCtrl), st) != cudaSuccess) return DP_ERR_CUDA;
     if (m > 0)
-      k_na_round<<<(int)(((int64_t)m + kNaThreads - 1) / kNaThreads), kNaThreads, 0, st>>>(
-          m, row_ptr, lhs, rhs, A);
+      k_na_round<<<(int)(((int64_t)m + per - 1) / per), kNaThreads, 0, st>>>(m, per, row_ptr, lhs,
+                                                                            rhs, A);
     if (n > 0)
       k_na_finish<<<(int)((n + 255) / 256), 256, 0, st>>>(n, vartype, keys, lb_out, ub_out, ctrl,
                                                           p.eps_feas);
