@@ -85,6 +85,12 @@ int upload(dp_matrix *mat, const std::vector<T> &v, const T **out, cudaStream_t 
 
 using dp::is_device_ptr;
 
+// A round that is expected to change more than n / kMarkShare variables does
+// not mark their chunks, and the next one processes all of them: marking costs
+// an atomic per nonzero of the changed variables, and at that share every long
+// row is marked anyway.
+constexpr int32_t kMarkShare = 32;
+
 // Where a team (dp_team.cu) takes a problem instead of the graph's kernels or
 // the batched ones.  A team's rounds cost less (a cluster barrier instead of
 // three to five kernels) and its marking skips unchanged rows, but it has 16
@@ -475,6 +481,8 @@ int load_layout(dp_ctx *ctx, dp::HostLayout &H, const std::vector<int32_t> *row_
     }
     M.col_ptr = ptr;
     M.col_slot = slot;
+    S.mask = mat->team_mask;  // one call on a matrix at a time
+    S.touch = mat->team_touch;
     if (cudaMallocHost(&mat->h_res, sizeof(int4) * nflags) != cudaSuccess) {
       cudaGetLastError();
       dp_matrix_free(mat);
@@ -739,6 +747,8 @@ int begin_call(dp_ctx *ctx, dp_matrix *mat, const double *lb, const double *ub,
   dp::Ctrl *hc = ctx->h_ctrl;
   std::memset(hc, 0, sizeof(*hc));
   hc->max_rounds = p.max_rounds;
+  hc->all_active = 1;
+  hc->mark_limit = mat->M.col_ptr ? n / kMarkShare : -1;
   hc->eps_int = p.eps_int;
   hc->tau_rel = p.tau_rel;
   hc->eps_feas = p.eps_feas;

@@ -112,6 +112,12 @@ struct Ctrl {
   int32_t qcount;       // entries appended to the candidate queue this round
   int32_t cont;         // the last round asked for another one
   int32_t pad;
+  int32_t all_active;   // this round processes every chunk, not only the marked ones
+  int32_t all_next;     // the commit left a variable of too many rows unmarked
+  int32_t nchanged;     // variables committed this round
+  int32_t mark_now;     // this round's commit marks the changed variables' chunks
+  int32_t mark_limit;   // most changed variables to mark one by one (-1: never)
+  int32_t pad2;
   double eps_int, tau_rel, eps_feas, inf_thr;
   long long wait_limit;  // persistent loop: sleeps a block waits at a grid barrier
 };
@@ -193,6 +199,9 @@ struct DevState {
   uint32_t *mp_need;    // merge path: [ceil(mp_nseg/32)] activities a warp's rows need
   Ctrl *ctrl;
   uint32_t *dirty;      // [ceil(n/32)] bit j: x_j's next state changed this round
+  uint32_t *mask;       // [nslices] chunks of each slice with a variable that changed in
+                        // the previous round (read and cleared by the round)
+  int32_t *touch;       // [nsplit_rows] last round that recomputed a piece of the row
   unsigned *bar;        // [2] grid barrier of the persistent loop: arrivals, generation
   InstState I;          // problem sets only
 };

@@ -312,6 +312,68 @@ __device__ __forceinline__ bool warp_enqueue(const RowView &mine, const Top2 &t,
   return full;
 }
 
+// ---- marking ----
+
+// Position of the k-th set bit (k from 0) of a word that has more than k.
+__device__ __forceinline__ int nth_bit(uint32_t w, int k) {
+  int at = 0;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const int c = __popc((w >> at) & ((1u << o) - 1u));
+    if (k >= c) {
+      k -= c;
+      at += o;
+    }
+  }
+  return at;
+}
+
+// Marks the chunks of the lanes' variables (deg list entries each from beg;
+// deg = 0 for none): the lists are walked as one sequence, so that the lanes
+// stay busy whatever the column lengths.  A mask only gains bits while a
+// round is committed, so a word that is seen, possibly in an older state, to
+// have the bit needs no atomic.  kCo: the masks are read through L2 (needed
+// where L1 may hold a word of an earlier round).  All 32 lanes call.
+template <bool kCo>
+__device__ __forceinline__ void mark_columns(const int32_t *col_slot, uint32_t *mask, int32_t beg,
+                                             int32_t deg) {
+  const int lane = threadIdx.x & 31;
+  int32_t incl = deg;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int32_t v = __shfl_up_sync(kFull, incl, o);
+    if (lane >= o) incl += v;
+  }
+  const int32_t total = __shfl_sync(kFull, incl, 31);
+  const int32_t shift = beg - (incl - deg);  // list offset of sequence position 0
+  for (int32_t e0 = 0; e0 < total; e0 += 128) {
+    int32_t slot[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int32_t e = e0 + 32 * u + lane;
+      int src = 0;  // the variable whose list holds position e
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const int32_t v = __shfl_sync(kFull, incl, src + o - 1);
+        if (v <= e) src += o;
+      }
+      const int32_t sh = __shfl_sync(kFull, shift, src & 31);
+      slot[u] = e < total ? __ldg(col_slot + e + sh) : -1;
+    }
+    uint32_t w[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const uint32_t *q = mask + (slot[u] >> 5);
+      w[u] = slot[u] < 0 ? 0u : (kCo ? __ldcg(q) : __ldca(q));
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const uint32_t bit = 1u << (slot[u] & 31);
+      if (slot[u] >= 0 && !(w[u] & bit)) atomicOr(mask + (slot[u] >> 5), bit);
+    }
+  }
+}
+
 // Appends one queue entry per lane with h set (warp-aggregated; all 32
 // lanes call): element offset `off` of a row whose sums are at rowsum[slot].
 __device__ __forceinline__ void warp_push(bool h, int64_t off, int64_t slot, unsigned sides,

@@ -805,60 +805,6 @@ constexpr int32_t kMarkAlways = 1 << 15;  // fewer variables: always marked
 constexpr int32_t kMarkDegree = 4096;     // more rows than this: every chunk
 constexpr int kCommitWords = 8;           // most dirty words per warp and step
 
-// Position of the k-th set bit (k from 0) of a word that has more than k.
-__device__ __forceinline__ int nth_bit(uint32_t w, int k) {
-  int at = 0;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const int c = __popc((w >> at) & ((1u << o) - 1u));
-    if (k >= c) {
-      k -= c;
-      at += o;
-    }
-  }
-  return at;
-}
-
-// Marks the chunks of the lanes' variables (deg list entries each from beg;
-// deg = 0 for none): the lists are walked as one sequence, so that the lanes
-// stay busy whatever the column lengths.  All 32 lanes call.
-__device__ __forceinline__ void mark_columns(const TeamArgs &A, const Team &T, int32_t beg,
-                                             int32_t deg) {
-  const int lane = threadIdx.x & 31;
-  int32_t incl = deg;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int32_t v = __shfl_up_sync(kFull, incl, o);
-    if (lane >= o) incl += v;
-  }
-  const int32_t total = __shfl_sync(kFull, incl, 31);
-  uint32_t *mask = T.mask + (T.p ^ 1) * T.nmask;
-  const int32_t shift = beg - (incl - deg);  // list offset of sequence position 0
-  for (int32_t e0 = 0; e0 < total; e0 += 128) {
-    int32_t slot[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int32_t e = e0 + 32 * u + lane;
-      int src = 0;  // the variable whose list holds position e
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const int32_t v = __shfl_sync(kFull, incl, src + o - 1);
-        if (v <= e) src += o;
-      }
-      const int32_t sh = __shfl_sync(kFull, shift, src & 31);
-      slot[u] = e < total ? __ldg(A.M.col_slot + e + sh) : -1;
-    }
-    uint32_t w[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) w[u] = slot[u] >= 0 ? __ldcg(mask + (slot[u] >> 5)) : 0u;
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const uint32_t bit = 1u << (slot[u] & 31);
-      if (slot[u] >= 0 && !(w[u] & bit)) atomicOr(mask + (slot[u] >> 5), bit);
-    }
-  }
-}
-
 // Ends a round: the changed variables' keys become their records, crossing
 // bounds are infeasible, and the variables' chunks are marked for the next
 // round.  A warp takes kCommitWords words of the dirty bitmap and then their
@@ -928,7 +874,7 @@ __device__ __noinline__ void commit_round(const TeamArgs &A, const Team &T, floa
       if (__any_sync(kFull, deg > kMarkDegree)) {
         if (lane == 0) T.flags->all_next[T.p] = 1;
       } else if (mark) {
-        mark_columns(A, T, beg, deg);
+        mark_columns<true>(A.M.col_slot, T.mask + (T.p ^ 1) * T.nmask, beg, deg);
       }
     }
   }
