@@ -457,6 +457,27 @@ int load_layout(dp_ctx *ctx, dp::HostLayout &H, const std::vector<int32_t> *row_
   // candidate queue: at most one entry per slot and round, so it never
   // overflows; row sums are stored per chunk slot
   TRY(dev_alloc(mat, &S.queue, (size_t)mat->padded));
+  {
+    // the queues' room: the slots of their slices (merge path: the nonzeros of
+    // every 32 rows in the layout's order)
+    std::vector<uint32_t> qbase(dp::kQueues, 0);
+    std::vector<int64_t> room(dp::kQueues, 0);
+    for (int32_t q = 0; q < H.nslices; ++q)
+      for (int t = 0; t < dp::kSliceW; ++t)
+        room[(size_t)(q % dp::kQueues)] +=
+            H.chunk_len[(size_t)q * dp::kSliceW + (size_t)t] & dp::kLenMask;
+    for (size_t q = 1; q < qbase.size(); ++q)
+      qbase[q] = (uint32_t)(qbase[q - 1] + room[q - 1]);
+    TRY(upload(mat, qbase, &S.qbase, st));
+    TRY(dev_alloc(mat, &S.qcount, (size_t)dp::kQueues * dp::kQueueStep));
+    if (cudaMemsetAsync(S.qcount, 0, sizeof(int32_t) * dp::kQueues * dp::kQueueStep, st) !=
+            cudaSuccess ||
+        cudaStreamSynchronize(st) != cudaSuccess) {  // qbase is a local
+      cudaGetLastError();
+      dp_matrix_free(mat);
+      return DP_ERR_CUDA;
+    }
+  }
   TRY(dev_alloc(mat, &S.rowsum, (size_t)H.nslices * dp::kSliceW));
   TRY(dev_alloc(mat, &S.side, (size_t)H.nslices * dp::kSliceW));
   TRY(dev_alloc(mat, &S.ctrl, 1));

@@ -87,7 +87,10 @@ struct alignas(16) RowTot {
 // One nonzero whose candidates survived the screen, queued for the
 // lane-dense candidate kernel: its element offset in val/col, and
 // (chunk slot << 2 | sides), sides bit 0 = right-hand side, bit 1 = left.
-// The queue holds one entry per slot at most, so it cannot overflow.
+// The queue is kQueues queues (slice s appends to queue s % kQueues), each with
+// room for every slot of its slices, so none can overflow.  With a single
+// one the appends of a round, one returning atomic per slice and more,
+// queued up at its counter: 1.2 ns each, for 65,000 slices 80 us.
 struct alignas(8) CandEntry {
   uint32_t off;
   uint32_t cs;
@@ -100,6 +103,9 @@ struct alignas(8) RowSum {
   int32_t mininf, maxinf;
 };
 
+constexpr int kQueues = 64;
+constexpr int kQueueStep = 32;  // words between the counters: a line each
+
 // Device control block of one propagation run.
 struct Ctrl {
   int32_t round;        // executed rounds
@@ -109,7 +115,7 @@ struct Ctrl {
   int32_t infeasible;
   int32_t err;          // 0, or a DP_ERR_* code found by the prologue
   uint32_t blocks_done; // arrival counter of the last kernel of a round
-  int32_t qcount;       // entries appended to the candidate queue this round
+  int32_t pad0;
   int32_t cont;         // the last round asked for another one
   int32_t pad;
   int32_t all_active;   // this round processes every chunk, not only the marked ones
@@ -187,7 +193,9 @@ struct InstState {
 };
 
 struct DevState {
-  CandEntry *queue;     // [padded slots] candidate queue
+  CandEntry *queue;     // [padded slots] candidate queues, one behind the other
+  int32_t *qcount;      // [kQueues * kQueueStep] entries of each this round
+  const uint32_t *qbase;  // [kQueues] first entry of each
   RowSum *rowsum;       // [chunk slots] sums of rows with queued nonzeros
   VarRec *rec;          // [n] state at the start of the round
   long long *keys;      // [2n] next state as order-preserving int64 keys

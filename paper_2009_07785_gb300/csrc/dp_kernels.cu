@@ -48,11 +48,10 @@ namespace dp {
 // round (L, U).  A variable that receives a candidate is marked in the
 // round's dirty bitmap; the atomics return nothing, so none of them waits
 // for its answer.
-__device__ __forceinline__ void nnz_candidates(double a, int32_t j, double L, double U,
+__device__ __forceinline__ bool nnz_candidates(double a, int32_t j, double L, double U,
                                                uint32_t flags, unsigned sides,
                                                const RowView &rv, const Ctrl &prm,
-                                               long long *keys, uint32_t *dirty,
-                                               int32_t *changed) {
+                                               long long *keys, uint32_t *dirty) {
   const bool isint = (flags & 1u) != 0u;
   bool any = false;
   auto apply = [&](const SideCand &c) {
@@ -65,84 +64,83 @@ __device__ __forceinline__ void nnz_candidates(double a, int32_t j, double L, do
                        prm.inf_thr));
   if (sides == 3u)  // both sides: the left-hand one too
     apply(side_candidate(a, L, U, isint, false, rv, prm.eps_int, prm.tau_rel, prm.inf_thr));
-  if (any) {
-    atomicOr(&dirty[j >> 5], 1u << (j & 31));
-    *changed = 1;
-  }
+  if (any) atomicOr(&dirty[j >> 5], 1u << (j & 31));
+  return any;
 }
 
 // ---------------------------------------------------------- k_cand_queue --
 
-// One queued nonzero's operands: the entry, its row's sums and sides, its
-// coefficient and column, and the start-of-round record of its variable.
-struct QueuedNnz {
-  CandEntry E;
-  RowSum rs;
-  double2 sd;
-  double a;
-  int32_t j;
+// Evaluates one queued nonzero.  Returns whether a candidate was applied
+// (single problems: the caller sets the change flag; a set's problem's is set
+// here).
+template <bool kMulti, bool kCo = false>
+__device__ __forceinline__ bool cand_entry_eval(const DevMatrix &M, const DevState &S,
+                                                const Ctrl &prm, const CandEntry &E) {
+  const uint32_t c = E.cs >> 2;
+  const RowSum rs = S.rowsum[c];
+  const double2 sd = S.side[c];
+  const double a = ld_coef(M, E.off);
+  const int32_t j = M.col[E.off];
   double L, U;
   float WU, WL;
   uint32_t fl;
-};
-
-// Evaluates kN queued nonzeros per thread (entries e0 + u*stride, u < kN,
-// those below cnt): every load of one dependence level is issued for all
-// of them before the next level, so kN chains are in flight at once.
-template <bool kMulti, int kN, bool kCo = false>
-__device__ __forceinline__ void cand_entries(const DevMatrix &M, const DevState &S,
-                                             const Ctrl &prm, int64_t e0, int64_t stride,
-                                             int32_t cnt) {
-  QueuedNnz q[kN];
-  bool ok[kN];
-#pragma unroll
-  for (int u = 0; u < kN; ++u) {
-    ok[u] = e0 + u * stride < cnt;
-    if (ok[u]) q[u].E = S.queue[e0 + u * stride];
+  ld_rec_t<kCo>(S.rec + j, L, U, WU, WL, fl);
+  RowView rv;
+  rv.minfin = rs.minfin;
+  rv.maxfin = rs.maxfin;
+  rv.mininf = rs.mininf;
+  rv.maxinf = rs.maxinf;
+  rv.lhs = sd.x;
+  rv.rhs = sd.y;
+  rv.thr_r = rv.thr_l = f_inf();
+  rv.exact = 0;
+  rv.act = 1;
+  const bool any = nnz_candidates(a, j, L, U, fl, E.cs & 3u, rv, prm, S.keys, S.dirty);
+  if (kMulti && any) {
+    int32_t *f = &S.I.changed[S.I.slot_inst[c]];
+    if (__ldca(f) == 0) *f = 1;  // the flags share lines that every store would queue at
   }
-#pragma unroll
-  for (int u = 0; u < kN; ++u) {
-    if (!ok[u]) continue;
-    const uint32_t c = q[u].E.cs >> 2;
-    q[u].rs = S.rowsum[c];
-    q[u].sd = S.side[c];
-    q[u].a = ld_coef(M, q[u].E.off);
-    q[u].j = M.col[q[u].E.off];
-  }
-#pragma unroll
-  for (int u = 0; u < kN; ++u)
-    if (ok[u]) ld_rec_t<kCo>(S.rec + q[u].j, q[u].L, q[u].U, q[u].WU, q[u].WL, q[u].fl);
-#pragma unroll
-  for (int u = 0; u < kN; ++u) {
-    if (!ok[u]) continue;
-    const uint32_t c = q[u].E.cs >> 2;
-    RowView rv;
-    rv.minfin = q[u].rs.minfin;
-    rv.maxfin = q[u].rs.maxfin;
-    rv.mininf = q[u].rs.mininf;
-    rv.maxinf = q[u].rs.maxinf;
-    rv.lhs = q[u].sd.x;
-    rv.rhs = q[u].sd.y;
-    rv.thr_r = rv.thr_l = f_inf();
-    rv.exact = 0;
-    rv.act = 1;
-    int32_t *changed = kMulti ? &S.I.changed[S.I.slot_inst[c]] : &S.ctrl->changed;
-    nnz_candidates(q[u].a, q[u].j, q[u].L, q[u].U, q[u].fl, q[u].E.cs & 3u, rv, prm, S.keys,
-                   S.dirty, changed);
-  }
+  return any;
 }
 
-// Evaluates the queued nonzeros, one per thread and step (grid-stride; the
-// grid is sized to the blocks that fit on the GPU at once).
+// Evaluates the queued nonzeros, one per thread and step, the blocks dealt out
+// to the queues (block-level).  Returns whether this thread applied a candidate.
+template <bool kMulti, bool kCo>
+__device__ __forceinline__ bool cand_queues(const DevMatrix &M, const DevState &S,
+                                            const Ctrl &prm) {
+  bool any = false;
+  const int nb = (int)gridDim.x;
+  for (int q = (int)blockIdx.x % kQueues; q < kQueues; q += nb) {  // once, unless blocks are few
+    const int32_t *n = S.qcount + q * kQueueStep;
+    const int32_t cnt = kCo ? __ldcg(n) : *n;
+    const CandEntry *queue = S.queue + S.qbase[q];
+    const int peers = nb > q ? (nb - q + kQueues - 1) / kQueues : 1;  // blocks of this queue
+    for (int64_t e = (int64_t)(blockIdx.x / kQueues) * blockDim.x + threadIdx.x; e < cnt;
+         e += (int64_t)peers * blockDim.x) {
+      CandEntry E;
+      if (kCo) {
+        const long long w = __ldcg(reinterpret_cast<const long long *>(queue + e));
+        E.off = (uint32_t)w;
+        E.cs = (uint32_t)((unsigned long long)w >> 32);
+      } else {
+        E = queue[e];
+      }
+      any |= cand_entry_eval<kMulti, kCo>(M, S, prm, E);
+    }
+  }
+  return any;
+}
+
+// The grid is sized to the blocks that fit on the GPU at once.  One store per
+// block sets the change flag: with one per accepted candidate the early
+// rounds waited for its line.
 template <bool kMulti>
 __global__ void __launch_bounds__(256) k_cand_queue(DevMatrix M, DevState S) {
   const Ctrl *ctrl = S.ctrl;
   if (ctrl->err) return;
-  const int32_t cnt = ctrl->qcount;
   const Ctrl prm = *ctrl;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < cnt; e += stride)
-    cand_entries<kMulti, 1>(M, S, prm, e, stride, cnt);
+  const bool any = cand_queues<kMulti, false>(M, S, prm);
+  if (!kMulti && __syncthreads_or(any) && threadIdx.x == 0) S.ctrl->changed = 1;
 }
 
 // ------------------------------------------------------------- k_round --
@@ -359,7 +357,7 @@ __device__ __forceinline__ void short_rows(const DevMatrix &M, const DevState &S
     }
   }
   uint32_t m = mr | ml;
-  int pos = warp_reserve<4>(__popc(m), &S.ctrl->qcount);
+  uint32_t pos = warp_reserve<4>(__popc(m), c, S);
   if (m == 0u) return;
   RowSum rs;
   rs.minfin = rv.minfin;
@@ -1263,6 +1261,7 @@ __device__ __forceinline__ int decide_round(const DevState &S) {
   volatile Ctrl *vc = S.ctrl;
   const int32_t r = vc->round + 1;
   int32_t cont;
+  if (threadIdx.x < kQueues) S.qcount[threadIdx.x * kQueueStep] = 0;
   if (kMulti) {
     volatile int32_t *ch = S.I.changed, *inf = S.I.infeasible, *dn = S.I.done;
     int live = 0;
@@ -1293,7 +1292,6 @@ __device__ __forceinline__ int decide_round(const DevState &S) {
   if (threadIdx.x == 0) {
     vc->round = r;
     vc->changed = 0;
-    vc->qcount = 0;
     // The next round processes every chunk unless this one marked.  The next
     // round marks if it is expected to change few enough variables (rounds
     // change about three quarters of what the round before did).
@@ -1419,8 +1417,7 @@ k_persistent(DevMatrix M, DevState S, const uint8_t *vartype) {
       for (int sl = gw; sl < M.nslices_split; sl += nw) cand_split_slice<true>(M, S, sl);
       if (!grid_sync(S, lim)) return;
     }
-    const int32_t cnt = ((volatile Ctrl *)S.ctrl)->qcount;
-    for (int64_t e = gt; e < cnt; e += nt) cand_entries<kMulti, 1, true>(M, S, prm, e, nt, cnt);
+    if (cand_queues<kMulti, true>(M, S, prm) && !kMulti) S.ctrl->changed = 1;
     if (!grid_sync(S, lim)) return;
     const bool mark = ((volatile Ctrl *)S.ctrl)->mark_now != 0;
     const int64_t nwords = ((int64_t)M.n + 31) >> 5;
@@ -1513,6 +1510,7 @@ __global__ void k_prologue_sides(DevMatrix M, DevState S, const double *lhs, con
     }
     S.side[c] = make_double2(l, r);
   }
+  if (blockIdx.x == 0 && threadIdx.x < kQueues) S.qcount[threadIdx.x * kQueueStep] = 0;
   if (M.col_ptr == nullptr) return;
   // nothing is marked (the first round processes every chunk); an aborted
   // call may have left marks and touched rows behind

@@ -156,12 +156,13 @@ __device__ __forceinline__ uint32_t short_survivors(const float (&t)[kMax], int3
   return m & all;
 }
 
-// Reserves c (0..15) consecutive queue entries per lane with one atomic per
-// warp (all 32 lanes call): the lanes' offsets come from ballots of the bits
-// of c (kBits of them), not from a shuffle scan.  Returns the lane's first entry
+// Reserves c (0..15) consecutive entries per lane in the queue of chunk slots
+// slot..slot+31 with one atomic per warp (all 32 lanes call): the lanes'
+// offsets come from ballots of the bits of c (kBits of them), not from a
+// shuffle scan.  Returns the lane's first entry
 // (meaningless when c = 0).
 template <int kBits = 3>
-__device__ __forceinline__ int warp_reserve(int c, int32_t *counter) {
+__device__ __forceinline__ uint32_t warp_reserve(int c, int64_t slot, const DevState &S) {
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
   int total = 0, before = 0;
@@ -171,10 +172,13 @@ __device__ __forceinline__ int warp_reserve(int c, int32_t *counter) {
     total += __popc(b) << k;
     before += __popc(b & lt) << k;
   }
-  if (total == 0) return 0;
-  int base = 0;
-  if (lane == 0) base = atomicAdd(counter, total);
-  return __shfl_sync(kFull, base, 0) + before;
+  if (total == 0) return 0u;
+  uint32_t base = 0u;
+  if (lane == 0) {
+    const int q = (int)(slot >> 5) % kQueues;
+    base = S.qbase[q] + (uint32_t)atomicAdd(S.qcount + q * kQueueStep, total);
+  }
+  return __shfl_sync(kFull, base, 0) + (uint32_t)before;
 }
 
 // Queueing of the nonzeros of the lanes' chunks whose candidates survive
@@ -235,7 +239,7 @@ __device__ __forceinline__ bool enqueue_named(const RowView &mine, const Top2 &t
   }
   const bool merge = h1 && h2 && k1 == k2;
   const bool q2 = h2 && !merge;
-  int pos = warp_reserve((h1 ? 1 : 0) + (q2 ? 1 : 0), &S.ctrl->qcount);
+  uint32_t pos = warp_reserve((h1 ? 1 : 0) + (q2 ? 1 : 0), chunk_slot, S);
   if (h1 || q2 || full) put_rowsum(mine, chunk_slot, S);
   if (h1) S.queue[pos++] = cand_entry(elem0 + (int64_t)k1 * kStride, chunk_slot, merge ? 3u : 1u);
   if (q2) S.queue[pos] = cand_entry(elem0 + (int64_t)k2 * kStride, chunk_slot, 2u);
@@ -290,7 +294,7 @@ __device__ __forceinline__ void enqueue_reread(const RowView &mine, int32_t len,
     int c = 0;
 #pragma unroll
     for (int u = 0; u < 4; ++u) c += sd[u] != 0u;
-    int pos = warp_reserve(c, &S.ctrl->qcount);
+    uint32_t pos = warp_reserve(c, chunk_slot, S);
 #pragma unroll
     for (int u = 0; u < 4; ++u)
       if (sd[u] != 0u)
@@ -382,8 +386,11 @@ __device__ __forceinline__ void warp_push(bool h, int64_t off, int64_t slot, uns
   if (pm == 0u) return;
   const int lane = threadIdx.x & 31;
   const int leader = __ffs(pm) - 1;
-  int base = 0;
-  if (lane == leader) base = atomicAdd(&S.ctrl->qcount, __popc(pm));
+  uint32_t base = 0u;
+  if (lane == leader) {
+    const int q = (int)(slot >> 5) % kQueues;
+    base = S.qbase[q] + (uint32_t)atomicAdd(S.qcount + q * kQueueStep, __popc(pm));
+  }
   base = __shfl_sync(kFull, base, leader);
   if (!h) return;
   CandEntry e;
