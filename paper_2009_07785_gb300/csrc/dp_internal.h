@@ -123,7 +123,7 @@ struct Ctrl {
   int32_t nchanged;     // variables committed this round
   int32_t mark_now;     // this round's commit marks the changed variables' chunks
   int32_t mark_limit;   // most changed variables to mark one by one (-1: never)
-  int32_t pad2;
+  int32_t sparse;       // this round processes the chunks of very few variables
   double eps_int, tau_rel, eps_feas, inf_thr;
   long long wait_limit;  // persistent loop: sleeps a block waits at a grid barrier
 };

@@ -545,7 +545,6 @@ __device__ __forceinline__ RowView whole_row(const ChunkHead &h, const ChunkAcc 
 // row in CSR order, the same bits as round_slice, and the chain (about 64
 // clocks per slot: the binary64 pipe) is all that remains serial.
 constexpr int kTeamU = 2;            // slots per warp and step
-constexpr int kCoopMost = 3;         // marked chunks of a long slice up to which a warp takes them in turn
 constexpr int kTeamBlocksPerSM = 4;  // long slices per SM up to which a block takes each
 
 struct TeamPart {  // one warp's share of a chunk
@@ -837,39 +836,41 @@ __device__ __forceinline__ uint32_t take_mask(const DevState &S, int slice, bool
   return all ? kFull : __shfl_sync(kFull, m, 0);
 }
 
-// The first `teams` slices by a block each, the others by a warp each.
+// The nlong long slices first, the others by a warp each.  A block takes a
+// long slice when there are few of them (`few`) or very few chunks are marked
+// (30M nonzeros, 15 long slices per SM, 0.05% of the variables changed: 84 ->
+// 49 us; with 1% changed the blocks are slower, 171 -> 321 us); else it takes
+// kRoundWarps of them, and the blocks left over return.
 template <bool kMulti, int kRoundWarps, bool kVal8>
 __global__ void __launch_bounds__(kRoundWarps * 32, kRoundWarpsPerSM / kRoundWarps)
-k_round(DevMatrix M, DevState S, int teams) {
+k_round(DevMatrix M, DevState S, int few) {
   __shared__ TeamBuf<kRoundWarps> sb;
   __shared__ uint32_t s_bits;
   if (S.ctrl->err) return;
   const bool all = S.ctrl->all_active != 0;
-  if ((int)blockIdx.x < teams) {
-    const int slice = nth_slice(M, blockIdx.x);
-    if (threadIdx.x < 32) {
-      const uint32_t b = take_mask(S, slice, all);
-      if (threadIdx.x == 0) s_bits = b;
+  const int b = (int)blockIdx.x, warp = threadIdx.x >> 5;
+  if (b < M.nlong && (few || S.ctrl->sparse)) {
+    const int slice = nth_slice(M, b);
+    if (warp == 0) {
+      const uint32_t m = take_mask(S, slice, all);
+      if (threadIdx.x == 0) s_bits = m;
     }
     __syncthreads();
-    uint32_t b = s_bits;
-    if (__popc(b) <= kRoundWarps) {  // few chunks: one per warp
-      for (int at = 0; b != 0u; b &= b - 1u, ++at)
-        if (at == (int)(threadIdx.x >> 5)) coop_chunk<kMulti, kVal8>(M, S, slice, __ffs(b) - 1);
+    uint32_t m = s_bits;
+    if (__popc(m) <= kRoundWarps) {  // few chunks: one per warp
+      for (int at = 0; m != 0u; m &= m - 1u, ++at)
+        if (at == warp) coop_chunk<kMulti, kVal8>(M, S, slice, __ffs(m) - 1);
     } else {
-      team_slice<kMulti, kRoundWarps, kVal8>(M, S, slice, b, sb);
+      team_slice<kMulti, kRoundWarps, kVal8>(M, S, slice, m, sb);
     }
     return;
   }
-  const int q = teams + ((int)blockIdx.x - teams) * kRoundWarps + (threadIdx.x >> 5);
-  if (q >= M.nslices) return;  // warp-uniform
+  const int q = b < M.nlong ? b * kRoundWarps + warp
+                            : M.nlong + (b - M.nlong) * kRoundWarps + warp;
+  if (q >= (b < M.nlong ? M.nlong : M.nslices)) return;  // warp-uniform
   const int slice = nth_slice(M, q);
-  uint32_t bits = take_mask(S, slice, all);
+  const uint32_t bits = take_mask(S, slice, all);
   if (bits == 0u) return;
-  if (q < M.nlong && __popc(bits) <= kCoopMost) {
-    for (; bits != 0u; bits &= bits - 1u) coop_chunk<kMulti, kVal8>(M, S, slice, __ffs(bits) - 1);
-    return;
-  }
   if (!kVal8 && q >= M.short0) short_slice<kMulti>(M, S, slice, bits);
   else round_slice<kMulti, kVal8>(M, S, slice, bits);
 }
@@ -1296,6 +1297,7 @@ __device__ __forceinline__ int decide_round(const DevState &S) {
     // round marks if it is expected to change few enough variables (rounds
     // change about three quarters of what the round before did).
     vc->all_active = vc->all_next || !vc->mark_now;
+    vc->sparse = vc->mark_now && !vc->all_next && vc->nchanged <= vc->mark_limit / 32;
     vc->all_next = 0;
     const int32_t nch = vc->nchanged;
     vc->nchanged = 0;
@@ -1570,14 +1572,14 @@ template <bool kMulti, int kRoundWarps>
 cudaError_t launch_ell_front(const DevMatrix &M, const DevState &S, int num_sms,
                              cudaStream_t st, cudaEvent_t *ev) {
   cudaError_t e;
-  const int teams = team_blocks(M, num_sms);
-  int nb = teams + (M.nslices - teams + kRoundWarps - 1) / kRoundWarps;
+  const int few = M.nlong <= kTeamBlocksPerSM * num_sms;
+  int nb = M.nlong + (M.nslices - M.nlong + kRoundWarps - 1) / kRoundWarps;
   if (nb < 1) nb = 1;
   if (ev) cudaEventRecord(ev[0], st);
   if (M.val8)
-    k_round<kMulti, kRoundWarps, true><<<nb, kRoundWarps * 32, 0, st>>>(M, S, teams);
+    k_round<kMulti, kRoundWarps, true><<<nb, kRoundWarps * 32, 0, st>>>(M, S, few);
   else
-    k_round<kMulti, kRoundWarps, false><<<nb, kRoundWarps * 32, 0, st>>>(M, S, teams);
+    k_round<kMulti, kRoundWarps, false><<<nb, kRoundWarps * 32, 0, st>>>(M, S, few);
   if (ev) cudaEventRecord(ev[1], st);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (M.nsplit_rows > 0) {
