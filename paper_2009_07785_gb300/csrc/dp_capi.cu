@@ -318,8 +318,10 @@ void dp_destroy(dp_ctx *ctx) {
 namespace {
 void free_batch(BatchWs *b) {
   if (!b) return;
-  if (b->exec) cudaGraphExecDestroy(b->exec);
-  if (b->graph) cudaGraphDestroy(b->graph);
+  for (int k = 0; k < 2; ++k) {
+    if (b->exec[k]) cudaGraphExecDestroy(b->exec[k]);
+    if (b->graph[k]) cudaGraphDestroy(b->graph[k]);
+  }
   for (void *p : b->allocs) dp::dev_free(p);
   if (b->h_ctrl) cudaFreeHost(b->h_ctrl);
   if (b->h_nodes) cudaFreeHost(b->h_nodes);
@@ -1213,17 +1215,24 @@ int ensure_batch(dp_matrix *mat, int32_t Bp) {
     return DP_ERR_OOM;
   }
   b->Bp_cap = Bp;
-  const int sms = mat->ctx->num_sms;
-  const dp::DevMatrix Mc = mat->M;
-  const dp::BatchState Sc = b->S;
-  BTRY(build_loop_graph(
-      [Mc, Sc, sms](cudaGraphConditionalHandle h, cudaStream_t cs) {
-        return dp::launch_batch_round(Mc, Sc, h, 1, sms, cs, nullptr);
-      },
-      &b->graph, &b->exec));
 #undef BTRY
   mat->batch = b;
   return DP_OK;
+}
+
+// Makes (or reuses) the round loop of the workspace, `few` for a batch of
+// few nodes.
+int ensure_batch_graph(dp_matrix *mat, bool few) {
+  BatchWs *b = mat->batch;
+  if (b->exec[few]) return DP_OK;
+  const int sms = mat->ctx->num_sms;
+  const dp::DevMatrix Mc = mat->M;
+  const dp::BatchState Sc = b->S;
+  return build_loop_graph(
+      [Mc, Sc, sms, few](cudaGraphConditionalHandle h, cudaStream_t cs) {
+        return dp::launch_batch_round(Mc, Sc, h, 1, few, sms, cs, nullptr);
+      },
+      &b->graph[few], &b->exec[few]);
 }
 
 // Device copy of a host input (staged), or the device pointer itself.
@@ -1246,7 +1255,7 @@ int stage_in(BatchWs *b, T **slot, const T *src, size_t count, size_t cap, cudaS
 
 constexpr int kBatchStages = 6;  // mark, mark_split, act, combine, cand_split, finish
 
-int batch_hostloop(dp_matrix *mat, BatchWs *b, int32_t max_rounds, float *kernel_ms,
+int batch_hostloop(dp_matrix *mat, BatchWs *b, bool few, int32_t max_rounds, float *kernel_ms,
                    int32_t *kernel_launches) {
   dp_ctx *ctx = mat->ctx;
   cudaStream_t st = ctx->stream;
@@ -1262,7 +1271,7 @@ int batch_hostloop(dp_matrix *mat, BatchWs *b, int32_t max_rounds, float *kernel
   const bool launched[kBatchStages] = {true, split, true, split, split, true};
   int status = DP_OK;
   for (int32_t r = 0; r < max_rounds; ++r) {
-    cudaError_t e = dp::launch_batch_round(mat->M, b->S, 0, 0, ctx->num_sms, st,
+    cudaError_t e = dp::launch_batch_round(mat->M, b->S, 0, 0, few, ctx->num_sms, st,
                                            timed ? ev : nullptr);
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(b->h_ctrl, b->S.ctrl, sizeof(dp::BCtrl), cudaMemcpyDeviceToHost, st);
@@ -1417,6 +1426,14 @@ bool teams_for_nodes(const dp_ctx *ctx, const dp_matrix *mat, int32_t count) {
   return mat->M.nnz <= kTeamNodeNnz && mat->M.nnz * (int64_t)count <= kTeamNodeWork;
 }
 
+// Nodes up to which a batch's chunks share warps (k_bact_few).  Measured in us
+// per call (a chunk per warp / packed; random fixings and fixings at a point):
+// 2.0M nonzeros with rows of up to 20k: 8 nodes 692 / 447 and 5350 / 3626, 16 nodes
+// 755 / 601 and 5656 / 4540, 20 nodes 806 / 872 and 5828 / 6154, 32 nodes
+// 855 / 923 and 5918 / 6322; 1.2M nonzeros in short rows: 16 nodes 521 / 423 and
+// 3866 / 2961, 20 nodes 552 / 628 and 4017 / 4472.
+constexpr int32_t kFewNodes = 16;
+
 // How a dp_propagate_nodes call runs its rounds: the captured graph (a
 // WHILE loop of the round kernels), the host (one synchronisation per round,
 // so that each stage can be timed with CUDA events), or one persistent
@@ -1472,6 +1489,8 @@ int nodes_call(dp_ctx *ctx, const dp_matrix *cmat, int32_t count, const double *
     dp::TraceRange batch_range("node batch launch");
     const int32_t cnt = count - s0 < per ? count - s0 : per;
     const int32_t Bp = (cnt + 31) / 32 * 32;
+    const bool few = cnt <= kFewNodes;
+    if (p.max_rounds > 0 && mode == kNodesGraph && (rc = ensure_batch_graph(mat, few))) return rc;
     const size_t off = (size_t)s0 * (size_t)n, len = (size_t)cnt * (size_t)n;
     const double *d_lb = nullptr, *d_ub = nullptr;
     if ((rc = stage_in(b, &b->st_lb, n > 0 ? lb + off : lb, len, cap, st, &d_lb))) return rc;
@@ -1497,11 +1516,11 @@ int nodes_call(dp_ctx *ctx, const dp_matrix *cmat, int32_t count, const double *
     CUDA_TRY(dp::launch_batch_prologue(mat->M, b->S, cnt, d_lb, d_ub, d_vt, d_lhs, d_rhs,
                                        p.eps_int, p.tau_rel, p.eps_feas, p.inf_threshold,
                                        ctx->num_sms, st));
-    if (p.max_rounds > 0 && mode == kNodesGraph) CUDA_TRY(cudaGraphLaunch(b->exec, st));
+    if (p.max_rounds > 0 && mode == kNodesGraph) CUDA_TRY(cudaGraphLaunch(b->exec[few], st));
     if (p.max_rounds > 0 && mode == kNodesPersistent)
       CUDA_TRY(dp::launch_batch_persistent(mat->M, b->S, ctx->num_sms, st));
     if (p.max_rounds > 0 && mode == kNodesHostloop) {
-      int r2 = batch_hostloop(mat, b, p.max_rounds, kernel_ms, kernel_launches);
+      int r2 = batch_hostloop(mat, b, few, p.max_rounds, kernel_ms, kernel_launches);
       if (r2) return r2;
     }
     if (n > 0) {

@@ -304,10 +304,13 @@ struct BCtrl {
   int32_t err;        // 0, or a DP_ERR_* code found by the prologue
   int32_t any_alive;  // some node is still propagating
   uint32_t blocks_done;
+  uint32_t ticket;       // batches of work items handed out this round
   uint32_t bar_count;    // persistent loop: grid-barrier arrivals
   uint32_t bar_gen;      //   and its generation
   long long wait_limit;  // persistent loop: sleeps a block waits at a grid barrier
-  int32_t icount[kMaxGroups];  // work items of each node group this round
+  // work items of each node group this round: chunks of whole rows from the
+  // front of the group's region, chunks of split rows from its back
+  int32_t icount[kMaxGroups], scount[kMaxGroups];
   double eps_int, tau_rel, eps_feas, inf_thr;
 };
 
@@ -319,6 +322,7 @@ struct BatchState {
                         // (set while a round runs, committed and cleared after)
   uint32_t *cmask;      // [nslots*G] nodes of each group that process a chunk
   int32_t *items;       // [G*nslots] chunk slots to process, one region per group
+                        // (whole rows from its front, split rows from its back)
   BPartial *part;       // [nsplit_slots*Bp]
   BRowTot *rowtot;      // [nsplit_rows*Bp]
   uint32_t *srow_act;   // [nsplit_rows*G] nodes whose split row yields candidates

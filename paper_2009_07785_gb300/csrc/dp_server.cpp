@@ -219,7 +219,8 @@ int make_workspace(dp_server *s, Lane &L) {
   SRV_TRY(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
   cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeRelaxed);
   if (e == cudaSuccess) {
-    cudaError_t le = dp::launch_batch_round(L.mat->M, L.S, 0, 0, s->ctx->num_sms, cs, nullptr);
+    cudaError_t le = dp::launch_batch_round(L.mat->M, L.S, 0, 0, false, s->ctx->num_sms, cs,
+                                                nullptr);
     if (le == cudaSuccess)
       le = cudaMemcpyAsync(L.h_flags, L.S.node_done, 4 * (size_t)Bp, cudaMemcpyDeviceToHost, cs);
     if (le == cudaSuccess)
