@@ -98,16 +98,22 @@ constexpr int32_t kMarkShare = 32;
 //   one problem:  short rows 60k nonzeros 460 / 384, 179k 571 / 797;
 //                 irregular 60k 1112 / 634, 235k 1397 / 1275, 704k 2211 / 3790;
 //                 mixed 25k 1796 / 866, 126k 1750 / 1327, 378k 2187 / 2748
-//   nodes:        irregular 60k nonzeros, 33 nodes 1547 / 1073, 128 nodes
-//                 1974 / 2136; 235k, 8 nodes 2859 / 1474, 33 nodes 3783 / 2896,
-//                 128 nodes 5462 / 8902; 2.0M, 1 node 5717 / 6534;
-//                 short 24k, 128 nodes 1072 / 915, 256 nodes 1453 / 1494
+//   nodes:        irregular 60k nonzeros, 8 nodes 1296 / 705, 33 nodes
+//                 1560 / 1077, 100 nodes 1831 / 1825; 187k, 8 nodes 1694 / 1310
+//                 in many rounds but 188 / 233 in one, 16 nodes 1715 / 1991;
+//                 235k, 1 node 2445 / 1264 and 175 / 213;
+//                 short rows 60k, 8 nodes 678 / 456, 33 nodes 956 / 706,
+//                 100 nodes 1373 / 1707; 239k, 1 node 793 / 961, 16 nodes
+//                 1097 / 1639: without long chunks, which a team spreads over
+//                 its warps, the team's few blocks bound it sooner
 //   sets:         12 problems of up to 29k nonzeros 2855 / 842; 64 of up to
 //                 1.7M 8331 / 22885
-constexpr int64_t kTeamNnz = 100000;       // a single problem, or a set's largest
+constexpr int64_t kTeamNnz = 100000;       // a single problem, a set's largest, a node
+                                           // batch's matrix without long slices
 constexpr int64_t kTeamSetNnz = 4000000;   // a whole set
-constexpr int64_t kTeamNodeNnz = 300000;   // the matrix of a node batch
-constexpr int64_t kTeamNodeWork = 6000000; // its nonzeros times nodes
+constexpr int64_t kTeamNodeNnz = 300000;   // the matrix of a node batch with long slices
+constexpr int64_t kTeamNodeWork = 2500000;  // nonzeros times nodes: up to kTeamNnz nonzeros,
+constexpr int64_t kTeamNodeWorkLong = 1000000;  // and above
 constexpr int kTeamWarps = 8;  // warps per block of a team
 
 // Blocks of a team, a power of two: no more than give every slice a warp and
@@ -298,11 +304,13 @@ int dp_create(dp_ctx **out, int device, void *cuda_stream) {
     }
     ctx->own_stream = true;
   }
-  if (cudaMallocHost(&ctx->h_ctrl, sizeof(dp::Ctrl)) != cudaSuccess) {
+  // the results of teams first (16-byte aligned), the control block behind
+  if (cudaMallocHost(&ctx->h_res, sizeof(int4) + sizeof(dp::Ctrl)) != cudaSuccess) {
     if (ctx->own_stream) cudaStreamDestroy(ctx->stream);
     delete ctx;
     return DP_ERR_OOM;
   }
+  ctx->h_ctrl = reinterpret_cast<dp::Ctrl *>(ctx->h_res + 1);
   *out = ctx;
   return DP_OK;
 }
@@ -310,7 +318,7 @@ int dp_create(dp_ctx **out, int device, void *cuda_stream) {
 void dp_destroy(dp_ctx *ctx) {
   if (!ctx) return;
   cudaSetDevice(ctx->device);
-  if (ctx->h_ctrl) cudaFreeHost(ctx->h_ctrl);
+  if (ctx->h_res) cudaFreeHost(ctx->h_res);
   if (ctx->own_stream) cudaStreamDestroy(ctx->stream);
   delete ctx;
 }
@@ -346,8 +354,7 @@ void dp_matrix_free(dp_matrix *mat) {
   cudaStreamSynchronize(mat->ctx->stream);
   free_batch(mat->batch);
   free_teams(mat->teams);
-  if (mat->h_inst) cudaFreeHost(mat->h_inst);
-  if (mat->h_res) cudaFreeHost(mat->h_res);
+  if (mat->h_inst) cudaFreeHost(mat->h_res);  // a set's; else the context's
   if (mat->exec) cudaGraphExecDestroy(mat->exec);
   if (mat->graph) cudaGraphDestroy(mat->graph);
   for (void *p : mat->allocs) dp::dev_free(p);
@@ -459,10 +466,10 @@ int load_layout(dp_ctx *ctx, dp::HostLayout &H, const std::vector<int32_t> *row_
   // candidate queue: at most one entry per slot and round, so it never
   // overflows; row sums are stored per chunk slot
   TRY(dev_alloc(mat, &S.queue, (size_t)mat->padded));
+  // the queues' room: the slots of their slices (merge path: the nonzeros of
+  // every 32 rows in the layout's order)
+  std::vector<uint32_t> qbase(dp::kQueues, 0);
   {
-    // the queues' room: the slots of their slices (merge path: the nonzeros of
-    // every 32 rows in the layout's order)
-    std::vector<uint32_t> qbase(dp::kQueues, 0);
     std::vector<int64_t> room(dp::kQueues, 0);
     for (int32_t q = 0; q < H.nslices; ++q)
       for (int t = 0; t < dp::kSliceW; ++t)
@@ -470,15 +477,14 @@ int load_layout(dp_ctx *ctx, dp::HostLayout &H, const std::vector<int32_t> *row_
             H.chunk_len[(size_t)q * dp::kSliceW + (size_t)t] & dp::kLenMask;
     for (size_t q = 1; q < qbase.size(); ++q)
       qbase[q] = (uint32_t)(qbase[q - 1] + room[q - 1]);
-    TRY(upload(mat, qbase, &S.qbase, st));
-    TRY(dev_alloc(mat, &S.qcount, (size_t)dp::kQueues * dp::kQueueStep));
-    if (cudaMemsetAsync(S.qcount, 0, sizeof(int32_t) * dp::kQueues * dp::kQueueStep, st) !=
-            cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess) {  // qbase is a local
-      cudaGetLastError();
-      dp_matrix_free(mat);
-      return DP_ERR_CUDA;
-    }
+  }
+  TRY(upload(mat, qbase, &S.qbase, st));
+  TRY(dev_alloc(mat, &S.qcount, (size_t)dp::kQueues * dp::kQueueStep));
+  if (cudaMemsetAsync(S.qcount, 0, sizeof(int32_t) * dp::kQueues * dp::kQueueStep, st) !=
+      cudaSuccess) {
+    cudaGetLastError();
+    dp_matrix_free(mat);
+    return DP_ERR_CUDA;
   }
   TRY(dev_alloc(mat, &S.rowsum, (size_t)H.nslices * dp::kSliceW));
   TRY(dev_alloc(mat, &S.side, (size_t)H.nslices * dp::kSliceW));
@@ -506,11 +512,7 @@ int load_layout(dp_ctx *ctx, dp::HostLayout &H, const std::vector<int32_t> *row_
     M.col_slot = slot;
     S.mask = mat->team_mask;  // one call on a matrix at a time
     S.touch = mat->team_touch;
-    if (cudaMallocHost(&mat->h_res, sizeof(int4) * nflags) != cudaSuccess) {
-      cudaGetLastError();
-      dp_matrix_free(mat);
-      return DP_ERR_OOM;
-    }
+    mat->h_res = ctx->h_res;
   }
   TRY(dev_alloc(mat, &mat->vt_ws, (size_t)n));
   TRY(dev_alloc(mat, &mat->st_lb, (size_t)n));
@@ -547,11 +549,15 @@ int load_layout(dp_ctx *ctx, dp::HostLayout &H, const std::vector<int32_t> *row_
     TRY(dev_alloc(mat, &mat->team_next, 1));
     mat->row_off = *row_off;
     mat->var_off = *var_off;
-    if (cudaMallocHost(&mat->h_inst, sizeof(int32_t) * 3 * (size_t)count) != cudaSuccess) {
+    int4 *pinned = nullptr;
+    if (cudaMallocHost(&pinned, (sizeof(int4) + 3 * sizeof(int32_t)) * (size_t)count) !=
+        cudaSuccess) {
       cudaGetLastError();
       dp_matrix_free(mat);
       return DP_ERR_OOM;
     }
+    mat->h_res = pinned;
+    mat->h_inst = reinterpret_cast<int32_t *>(pinned + count);
   }
   if (cudaStreamSynchronize(st) != cudaSuccess) {
     cudaGetLastError();
@@ -1423,7 +1429,9 @@ int nodes_by_teams(dp_ctx *ctx, dp_matrix *mat, int32_t count, const double *lb,
 // Whether a team per node beats the batched kernels.
 bool teams_for_nodes(const dp_ctx *ctx, const dp_matrix *mat, int32_t count) {
   if (!mat->h_res || ctx->teams_of[0] <= 0) return false;
-  return mat->M.nnz <= kTeamNodeNnz && mat->M.nnz * (int64_t)count <= kTeamNodeWork;
+  const int64_t nnz = mat->M.nnz, work = nnz * (int64_t)count;
+  if (nnz <= kTeamNnz) return work <= kTeamNodeWork;
+  return mat->M.nlong > 0 && nnz <= kTeamNodeNnz && work <= kTeamNodeWorkLong;
 }
 
 // Nodes up to which a batch's chunks share warps (k_bact_few).  Measured in us

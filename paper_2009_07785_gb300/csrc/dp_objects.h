@@ -13,6 +13,7 @@ struct dp_ctx {
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   dp::Ctrl *h_ctrl = nullptr;  // pinned mirror of the device control block
+  int4 *h_res = nullptr;       // pinned, beside it: a single problem's team results
   int teams_of[5] = {0, 0, 0, 0, 0};  // teams of 1, 2, 4, 8, 16 blocks that fit at once
   int live_matrices = 0;
   long long wait_limit = dp::kDefaultWaitLimit;  // grid-barrier wait of the persistent loop
@@ -36,7 +37,7 @@ struct dp_matrix {
   dp::TeamFlags *team_flags = nullptr;
   uint32_t *team_mask = nullptr;   // [2 * nslices]
   int32_t *team_touch = nullptr;   // [split rows]
-  int4 *h_res = nullptr;           // pinned
+  int4 *h_res = nullptr;           // pinned: the context's, or a set's [ninst]
   // batched nodes (allocated on the first dp_propagate_nodes call)
   struct BatchWs *batch = nullptr;
   struct TeamWs *teams = nullptr;  // few nodes of a small matrix: a team each
@@ -44,7 +45,7 @@ struct dp_matrix {
   // problem sets (dp_matrix_load_set): first row / variable of each problem
   int32_t ninst = 0;
   std::vector<int32_t> row_off, var_off;
-  int32_t *h_inst = nullptr;  // pinned [3*ninst]: infeasible, rounds, status
+  int32_t *h_inst = nullptr;  // pinned [3*ninst], behind h_res: infeasible, rounds, status
   dp::TeamView *d_views = nullptr;  // [ninst] the problems, largest first
   int64_t largest = 0;              // nonzeros of the largest problem
   int32_t view_slices = 0;          // and its slices
