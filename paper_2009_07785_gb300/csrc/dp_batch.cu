@@ -30,9 +30,10 @@
 //                  variables); work lists per group
 //   k_bmark_split  block per split row: all chunks of a split row get the
 //                  row's mask
-//   k_bact         warp per work item: activities; for whole rows also
-//                  Step 2, the binary32 screen and the candidates with
-//                  filtered 64-bit atomics
+//   k_bact         warp per work item, handed out by ticket: activities; for
+//                  whole rows also Step 2, the binary32 screen and the
+//                  candidates with filtered 64-bit atomics (k_bact_few:
+//                  several work items of a batch of few nodes in a warp)
 //   k_bcombine     block per (split row, group): sums chunk partials in a
 //                  fixed order, Step 2 and screen thresholds
 //   k_bcand_split  warp per (split chunk, group): candidates of split rows

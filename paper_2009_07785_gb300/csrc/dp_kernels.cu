@@ -7,21 +7,27 @@
 //
 // Round structure (launched from a CUDA graph whose WHILE node repeats the
 // round until k_finish clears the condition -- no host round trip):
-//   k_round      one warp per slice, one lane per chunk: activities of every
-//                chunk (Def. 1, Eq. 2a/2b, Sec. 3.4 infinity counts); for
-//                whole rows also Step 2 and the binary32 screen, which
-//                queues the nonzeros whose candidates may be accepted
+//   k_round      one warp per slice, one lane per chunk (a block per long
+//                slice where few of them have work): activities of the
+//                round's chunks (Def. 1, Eq. 2a/2b, Sec. 3.4 infinity
+//                counts); for whole rows also Step 2 and the binary32
+//                screen, which queues the nonzeros whose candidates may be
+//                accepted
 //   k_combine    split rows of few pieces one per lane, rows of many pieces
 //                one per warp: sums the chunk partials in a fixed order,
 //                Step 2 and screen for the row
-//   k_cand_split one lane per chunk of an active split row: queueing
+//   k_cand_split one lane per chunk of an active split row (a block per long
+//                slice): queueing
 //   k_cand_queue one thread per queued nonzero: the candidates (Eq. 3a/3b
 //                via Eq. 5a/5b) with filtered atomics (Sec. 3.5); marks the
 //                variables it updates in a dirty bitmap
 //   k_finish     one warp per 8 bitmap words, per marked variable (the
 //                warp together): decode the next state, crossing test
 //                (Sec. 1.1, remark after Step 3), write the record the next
-//                round gathers; the last block decides whether to loop
+//                round gathers, and, when few variables changed, mark the
+//                chunks that hold them: the next round skips the others (the
+//                constraint marking of Alg. 1); the last block decides
+//                whether to loop and whether the next round marks
 // (The merge-path layout replaces the first three by the kernels of
 // dp_merge.cu.)
 //
