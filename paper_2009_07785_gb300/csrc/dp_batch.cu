@@ -62,7 +62,11 @@ constexpr int kActWarps = 8;
 // fixings at a point 36.4 -> 30.2).  Two items to a ticket where every warp has
 // at least 32 of them, else one: the tickets come from one counter (0.8M of
 // them in a dense round; one item each 5.5 ms, four 4.3 but 34.1 at a point).
+// Fixed shares remain below 8 items per warp if no chunk has 64 nonzeros: they
+// are even there, and a ticket costs 1.2 ns on the counter (200 nodes over 30k
+// nonzeros in short rows 660 us per call, 680 with tickets).
 constexpr int kActItems = 2;
+constexpr int kTicketItems = 8, kTicketSlots = 64;
 
 struct BParams {
   int32_t Bp, G, Gs, round, max_rounds, err;
@@ -583,11 +587,14 @@ __device__ __forceinline__ void bact_body(const DevMatrix &M, const BatchState &
   uint32_t *chg_next = S.chg[p ^ 1];
   const int bs = max(1, min(kActItems, total / (16 * nw)));
   const int nb = (total + bs - 1) / bs;
+  // tickets only where shares can be uneven: many items, or long chunks
+  const bool tickets = nb > kTicketItems * nw || (nb > nw && M.max_slots >= kTicketSlots);
   int next = blockIdx.x * kActWarps + (threadIdx.x >> 5);
   while (next < nb) {
     int it = next * bs;
     const int end = min(total, it + bs);
-    if (nb > nw && lane == 0) next = nw + (int)atomicAdd(&ctrl->ticket, 1u);
+    if (!tickets) next += nw;
+    else if (lane == 0) next = nw + (int)atomicAdd(&ctrl->ticket, 1u);
     for (; it < end; ++it) {
       const int g = __popc(__ballot_sync(kFull, lane < P.G && it >= incl));
       const int64_t cs = item_of(S, g, it - __shfl_sync(kFull, excl, g),
@@ -628,7 +635,6 @@ __device__ __forceinline__ void bact_body(const DevMatrix &M, const BatchState &
       if (!__any_sync(kFull, go)) continue;
       chunk_candidates<kCo>(M, S, base, len, node, go, row, rv, P, pq, chg_next);
     }
-    if (nb <= nw) break;
     next = __shfl_sync(kFull, next, 0);
   }
   drain_pairs<kCo>(pq, M, S, P, chg_next);

@@ -407,7 +407,10 @@ int load_layout(dp_ctx *ctx, dp::HostLayout &H, const std::vector<int32_t> *row_
   if (H.layout == dp::kLayoutEll) {
     auto len = [&](int32_t q) { return H.slice_len[(size_t)q]; };
     auto is_short = [&](int32_t q) { return q >= H.nslices_split && len(q) <= dp::kShortRow; };
-    for (int32_t q = 0; q < H.nslices; ++q) M.nlong += len(q) >= dp::kLongSlots;
+    for (int32_t q = 0; q < H.nslices; ++q) {
+      M.nlong += len(q) >= dp::kLongSlots;
+      M.max_slots = std::max(M.max_slots, len(q));
+    }
     if (row_off) {
       order.resize((size_t)H.nslices);
       for (int32_t q = 0; q < H.nslices; ++q) order[(size_t)q] = q;

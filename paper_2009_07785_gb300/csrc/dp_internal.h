@@ -140,6 +140,7 @@ struct DevMatrix {
   const int32_t *order;     // [nslices] a set's slices in the order the round takes them,
                             // long ones first, whole short rows last (null: nth_slice)
   int32_t nlong;            // slices of kLongSlots slots and more
+  int32_t max_slots;        // slots of the longest slice
   int32_t short0;           // position in that order from which on all rows are
                             // whole and have kShortRow nonzeros at most
   const double *val;        // padded slot-major values
