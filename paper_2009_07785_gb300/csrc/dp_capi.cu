@@ -1439,7 +1439,7 @@ bool teams_for_nodes(const dp_ctx *ctx, const dp_matrix *mat, int32_t count) {
 
 // Nodes up to which a batch's chunks share warps (k_bact_few).  Measured in us
 // per call (a chunk per warp / packed; random fixings and fixings at a point):
-// 2.0M nonzeros with rows of up to 20k: 8 nodes 692 / 447 and 5350 / 3626, 16 nodes
+// 2.0M nonzeros with knapsack rows: 8 nodes 692 / 447 and 5350 / 3626, 16 nodes
 // 755 / 601 and 5656 / 4540, 20 nodes 806 / 872 and 5828 / 6154, 32 nodes
 // 855 / 923 and 5918 / 6322; 1.2M nonzeros in short rows: 16 nodes 521 / 423 and
 // 3866 / 2961, 20 nodes 552 / 628 and 4017 / 4472.
