@@ -205,6 +205,7 @@ __device__ __forceinline__ void na_candidates(const NaArgs &A, const NaRow &r, d
 
 constexpr int kNaThreads = 256;
 constexpr int kNaWarps = kNaThreads / 32;
+constexpr int kNaBlocksPerSM = 3;  // resident blocks of k_na_round
 constexpr int kNaUnroll = 4;     // nonzeros whose loads are in flight together
 constexpr int kNaLaneRow = 32;   // longest row that one lane takes
 constexpr int kNaWarpRow = 256;  // longest row that one warp takes
@@ -359,7 +360,7 @@ __device__ __forceinline__ void na_row_block(const NaArgs &A, NaRow r, int64_t b
 // (two dependent loads and the binary64 chain), so a row of 12,000 nonzeros
 // took 12 ms per round where the block takes about 30 us.  A row of up to
 // kNaWarpRow nonzeros is one FMA chain in CSR order whichever way it goes.
-__global__ void __launch_bounds__(kNaThreads)
+__global__ void __launch_bounds__(kNaThreads, kNaBlocksPerSM)
 k_na_round(int32_t m, int per, const int64_t *row_ptr, const double *lhs_in,
            const double *rhs_in, NaArgs A) {
   __shared__ int s_long[kNaThreads];
@@ -540,8 +541,14 @@ extern "C" int dp_propagate_noalloc(int device, void *cuda_stream, int32_t m, in
   A.tau = p.tau_rel;
   A.eps_feas = p.eps_feas;
   A.thr = p.inf_threshold;
-  int per = 32;  // rows per block: about 600 blocks and more, four per SM
-  while (per < kNaThreads && m > 600 * per) per *= 2;
+  // rows per block: as few as leave every block resident at once.  A second wave
+  // of a few blocks costs as much as the first: 16k short rows in 511 blocks of
+  // 32 rows 1392 us per call, in 256 of 64 rows 955; 60k irregular ones in 469
+  // blocks 5278, in 235 4375.
+  int sms = 1, per = 32;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess)
+    return DP_ERR_CUDA;
+  while (per < kNaThreads && m > (int64_t)kNaBlocksPerSM * sms * per) per *= 2;
   int32_t r = 0;
   bool changed = false;
   for (; r < p.max_rounds;) {
