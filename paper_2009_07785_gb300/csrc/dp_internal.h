@@ -119,7 +119,7 @@ struct Ctrl {
   int32_t cont;         // the last round asked for another one
   int32_t pad;
   int32_t all_active;   // this round processes every chunk, not only the marked ones
-  int32_t all_next;     // the commit left a variable of too many rows unmarked
+  int32_t all_next;     // the commit left variables of too many rows unmarked
   int32_t nchanged;     // variables committed this round
   int32_t mark_now;     // this round's commit marks the changed variables' chunks
   int32_t mark_limit;   // most changed variables to mark one by one (-1: never)

@@ -1199,9 +1199,6 @@ __device__ __forceinline__ void finish_var(const DevState &S, const uint8_t *var
 
 constexpr int kFinishWords = 8;  // bitmap words per warp and step of k_finish
 
-// a variable in more rows than this is not marked by one warp either
-constexpr int32_t kMarkDegree = 4096;
-
 // Commits the variables marked in words [w0, w0 + kFinishWords) of the
 // dirty bitmap, clears those words and marks the variables' chunks for the
 // next round if `mark` (warp-level, all 32 lanes): lanes read one word each,
@@ -1249,7 +1246,7 @@ __device__ __forceinline__ int finish_words(const DevMatrix &M, const DevState &
       }
       finish_var<kMulti>(S, vartype, j, eps_feas, tau_dn, eps_dn);
     }
-    if (__any_sync(kFull, deg > kMarkDegree)) {
+    if (!markable(deg)) {
       if (lane == 0) S.ctrl->all_next = 1;
     } else if (mark) {
       mark_columns<kCo>(M.col_slot, S.mask, beg, deg);

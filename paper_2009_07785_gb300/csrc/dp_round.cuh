@@ -332,6 +332,18 @@ __device__ __forceinline__ int nth_bit(uint32_t w, int k) {
   return at;
 }
 
+// Whether the lists of the lanes' variables (deg entries each) are short enough
+// for the warp to walk; if not, the next round processes every chunk.  A walk
+// takes 0.25 us per 128 entries: without a limit the columns of a system with
+// few variables took longer than the rounds they saved (48 variables, 90k
+// nonzeros: 134 us per round, 20 with every chunk processed; a limit of 2048
+// entries leaves 500 variables at 510 us per call where 512 gives 385).
+// All 32 lanes call.
+constexpr int32_t kMarkEntries = 512;
+__device__ __forceinline__ bool markable(int32_t deg) {
+  return __reduce_add_sync(kFull, min(deg, kMarkEntries + 1)) <= kMarkEntries;
+}
+
 // Marks the chunks of the lanes' variables (deg list entries each from beg;
 // deg = 0 for none): the lists are walked as one sequence, so that the lanes
 // stay busy whatever the column lengths.  A mask only gains bits while a

@@ -802,7 +802,6 @@ __device__ __noinline__ int split_candidates(const TeamArgs &A, const Team &T, P
 // the changed variables, and at that share most rows are marked anyway.
 constexpr int kMarkShare = 12;
 constexpr int32_t kMarkAlways = 1 << 15;  // fewer variables: always marked
-constexpr int32_t kMarkDegree = 4096;     // more rows than this: every chunk
 constexpr int kCommitWords = 8;           // most dirty words per warp and step
 
 // Ends a round: the changed variables' keys become their records, crossing
@@ -871,7 +870,7 @@ __device__ __noinline__ void commit_round(const TeamArgs &A, const Team &T, floa
         }
         put_var(T.rec + j, L, U, isint, tau_dn, eps_dn);
       }
-      if (__any_sync(kFull, deg > kMarkDegree)) {
+      if (!markable(deg)) {
         if (lane == 0) T.flags->all_next[T.p] = 1;
       } else if (mark) {
         mark_columns<true>(A.M.col_slot, T.mask + (T.p ^ 1) * T.nmask, beg, deg);
