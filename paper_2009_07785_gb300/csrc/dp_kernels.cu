@@ -1263,7 +1263,10 @@ __device__ __forceinline__ int finish_words(const DevMatrix &M, const DevState &
 template <bool kMulti>
 __device__ __forceinline__ int decide_round(const DevState &S) {
   volatile Ctrl *vc = S.ctrl;
-  const int32_t r = vc->round + 1;
+  // every word before any decision, so that the loads overlap
+  const int32_t r = vc->round + 1, max_rounds = vc->max_rounds, err = vc->err;
+  const int32_t chg = vc->changed, infeasible = vc->infeasible, all_next = vc->all_next;
+  const int32_t mark_now = vc->mark_now, mark_limit = vc->mark_limit, nch = vc->nchanged;
   int32_t cont;
   if (threadIdx.x < kQueues) S.qcount[threadIdx.x * kQueueStep] = 0;
   if (kMulti) {
@@ -1276,7 +1279,7 @@ __device__ __forceinline__ int decide_round(const DevState &S) {
       int32_t d = 0;
       if (inf[i]) d = 1;
       else if (!ch[i]) d = 1;
-      else if (ri >= vc->max_rounds) {
+      else if (ri >= max_rounds) {
         d = 1;
         S.I.status[i] = 1;
       }
@@ -1285,11 +1288,10 @@ __device__ __forceinline__ int decide_round(const DevState &S) {
       live |= !d;
     }
     live = __syncthreads_or(live);
-    cont = (live && !vc->err && r < vc->max_rounds) ? 1 : 0;
+    cont = (live && !err && r < max_rounds) ? 1 : 0;
     if (threadIdx.x == 0) vc->last_changed = live;
   } else {
-    const int32_t chg = vc->changed;
-    cont = (chg && !vc->infeasible && !vc->err && r < vc->max_rounds) ? 1 : 0;
+    cont = (chg && !infeasible && !err && r < max_rounds) ? 1 : 0;
     __syncthreads();
     if (threadIdx.x == 0) vc->last_changed = chg;
   }
@@ -1299,12 +1301,12 @@ __device__ __forceinline__ int decide_round(const DevState &S) {
     // The next round processes every chunk unless this one marked.  The next
     // round marks if it is expected to change few enough variables (rounds
     // change about three quarters of what the round before did).
-    vc->all_active = vc->all_next || !vc->mark_now;
-    vc->sparse = vc->mark_now && !vc->all_next && vc->nchanged <= vc->mark_limit / 32;
+    const bool all = all_next || !mark_now;
+    vc->all_active = all;
+    vc->sparse = !all && nch <= mark_limit / 32;
     vc->all_next = 0;
-    const int32_t nch = vc->nchanged;
     vc->nchanged = 0;
-    vc->mark_now = nch - nch / 4 <= vc->mark_limit;
+    vc->mark_now = nch - nch / 4 <= mark_limit;
     vc->cont = cont;
     __threadfence();
   }
