@@ -417,8 +417,9 @@ int64_t dp_debug_live_allocs(void);
  * issued on `cuda_stream` (NULL = the legacy default stream); the host waits
  * for the stream after every round and the rounds have no screen and no
  * marking, so this path is for callers that cannot allocate, not the fast
- * path.  Rows of up to 256 nonzeros are summed in CSR order, longer ones by a
- * block's threads in a fixed order of their own.
+ * path.  Rows of up to 256 nonzeros are summed in CSR order, longer ones in
+ * CSR order or by a block's threads in a fixed order of their own (which of
+ * the two follows from m and the row lengths alone).
  *
  * Its only scratch -- the next-state bound keys and a control block -- is a
  * file-scope device array sized for n <= DP_NOALLOC_MAX_VARS variables

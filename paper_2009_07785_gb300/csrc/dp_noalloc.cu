@@ -209,6 +209,10 @@ constexpr int kNaBlocksPerSM = 3;  // resident blocks of k_na_round
 constexpr int kNaUnroll = 4;     // nonzeros whose loads are in flight together
 constexpr int kNaLaneRow = 32;   // longest row that one lane takes
 constexpr int kNaWarpRow = 256;  // longest row that one warp takes
+// What a row costs, in 0.062 us: a lane 2.1 us per nonzero (its candidates'
+// divisions, whatever the other lanes do), a warp 4 us and 0.062 us per nonzero, a
+// block 8 us and 0.012 us per nonzero.
+constexpr unsigned kNaLaneCost = 34, kNaWarpCost = 64, kNaBlockCost = 130, kNaBlockShare = 5;
 
 // Loads nonzeros k, k + step, ... (kNaUnroll of them, those below e).
 __device__ __forceinline__ void na_load(const NaArgs &A, int64_t k, int64_t step, int64_t e,
@@ -352,45 +356,73 @@ __device__ __forceinline__ void na_row_block(const NaArgs &A, NaRow r, int64_t b
   }
 }
 
-// One round, `per` rows (32..kNaThreads, a multiple of 32) per block: short
-// rows by a lane each, longer ones by a warp, the longest by the block.  Few
+// One round, `per` rows (32..kNaThreads, a multiple of 32) per block.  Few
 // rows are spread over as many blocks as there are, since the lanes' binary64
-// work shares one pipe per scheduler.  What bounds a round is the
-// latency of its longest row: one lane's walk takes about 1 us per nonzero
-// (two dependent loads and the binary64 chain), so a row of 12,000 nonzeros
-// took 12 ms per round where the block takes about 30 us.  A row of up to
-// kNaWarpRow nonzeros is one FMA chain in CSR order whichever way it goes.
+// work shares one pipe per scheduler.  What bounds a round is the latency of
+// the walks: rows of up to kNaLaneRow nonzeros go by a lane each, longer ones by
+// a warp and the longest by the block, one after the other, where that is shorter
+// than the longest one's walk by a lane (a row of 12,000 nonzeros takes 12 ms by
+// a lane, 30 us by the block; but 32 rows of 36 in a warp's turn 210 us by the
+// warp, 86 by the lanes).  A row of up to kNaWarpRow nonzeros is one FMA chain
+// in CSR order whichever way it goes.
 __global__ void __launch_bounds__(kNaThreads, kNaBlocksPerSM)
 k_na_round(int32_t m, int per, const int64_t *row_ptr, const double *lhs_in,
            const double *rhs_in, NaArgs A) {
+  const unsigned full = 0xFFFFFFFFu;
   __shared__ int s_long[kNaThreads];
   __shared__ int s_count;
-  if (threadIdx.x == 0) s_count = 0;
+  __shared__ unsigned s_rest;
+  __shared__ unsigned long long s_cost, s_top;
+  if (threadIdx.x == 0) {
+    s_count = 0;
+    s_rest = 0u;
+    s_cost = s_top = 0ull;
+  }
   __syncthreads();
   const int64_t i = blockIdx.x * (int64_t)per + threadIdx.x;
   NaRow r;
   r.minfin = r.maxfin = r.lhs = r.rhs = 0.0;
   r.mininf = r.maxinf = 0;
   int64_t b = 0, e = 0;
-  if (i < m && (int)threadIdx.x < per) {
+  const bool have = i < m && (int)threadIdx.x < per;
+  if (have) {
     r.lhs = side_norm(lhs_in[i], A.thr);
     r.rhs = side_norm(rhs_in[i], A.thr);
     b = row_ptr[i];
     e = row_ptr[i + 1];
-    if (e - b <= kNaLaneRow) na_row_lane(A, r, b, e);
-    else if (e - b > kNaWarpRow) s_long[atomicAdd(&s_count, 1)] = threadIdx.x;
   }
+  const unsigned long long len = (unsigned long long)(e - b);
+  if (len > kNaWarpRow) {
+    s_long[atomicAdd(&s_count, 1)] = threadIdx.x;
+    atomicAdd(&s_cost, kNaBlockCost + len / kNaBlockShare);
+    atomicMax(&s_top, len);
+  }
+  const unsigned most = __reduce_max_sync(full, len > kNaWarpRow ? 0u : (unsigned)len);
+  if ((threadIdx.x & 31) == 0) atomicMax(&s_rest, most);
+  __syncthreads();
+  // whether the block takes its long rows one after the other, or a lane each,
+  // which lengthens the lanes' walk
+  const bool by_block = s_cost < kNaLaneCost * (s_top - s_rest);
+  // the rows left to this warp: the mid ones by the warp one after the other, or
+  // by a lane each like the others
+  const unsigned wlen = len > kNaWarpRow && by_block ? 0u : (unsigned)min(len, 1ull << 26);
+  const bool mid = len > kNaLaneRow && len <= kNaWarpRow;
+  const unsigned rest = __reduce_max_sync(full, mid ? 0u : wlen);
+  const bool by_warp = kNaLaneCost * rest + __reduce_add_sync(full, mid ? kNaWarpCost + wlen : 0u) <
+                       kNaLaneCost * __reduce_max_sync(full, wlen);
+  if (have && !(mid && by_warp) && !(len > kNaWarpRow && by_block)) na_row_lane(A, r, b, e);
   __syncwarp();
-  unsigned todo = __ballot_sync(0xFFFFFFFFu, e - b > kNaLaneRow && e - b <= kNaWarpRow);
+  unsigned todo = __ballot_sync(full, mid && by_warp);
   for (; todo != 0u; todo &= todo - 1u) {
     const int src = __ffs(todo) - 1;
     NaRow q;
     q.minfin = q.maxfin = 0.0;
     q.mininf = q.maxinf = 0;
-    q.lhs = __shfl_sync(0xFFFFFFFFu, r.lhs, src);
-    q.rhs = __shfl_sync(0xFFFFFFFFu, r.rhs, src);
-    na_row_warp(A, q, __shfl_sync(0xFFFFFFFFu, b, src), __shfl_sync(0xFFFFFFFFu, e, src));
+    q.lhs = __shfl_sync(full, r.lhs, src);
+    q.rhs = __shfl_sync(full, r.rhs, src);
+    na_row_warp(A, q, __shfl_sync(full, b, src), __shfl_sync(full, e, src));
   }
+  if (!by_block) return;  // block-uniform
   __syncthreads();
   const int nlong = s_count;
   for (int q = 0; q < nlong; ++q) {  // block-uniform
