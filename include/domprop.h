@@ -472,8 +472,9 @@ int dp_propagate_noalloc(int device, void *cuda_stream, int32_t m, int32_t n,
  * allocates a workspace of about 80 bytes per (variable, node) pair kept
  * with the matrix (freed by dp_matrix_free); host inputs are staged.  Few
  * nodes of a small matrix run on a thread block cluster each instead, with a
- * workspace of about 50 bytes per variable and cluster; the results are the
- * same.
+ * workspace of about 50 bytes per variable and cluster and device buffers of up
+ * to 32 MB (or one bound vector per cluster, if that is more) for each of lb, ub,
+ * lb_out and ub_out that lies in host memory; the results are the same.
  * Returns DP_OK, DP_CAP_HIT (some node hit the cap), DP_ERR_INVALID_ARG,
  * DP_ERR_NAN_INPUT (any node), DP_ERR_OOM or DP_ERR_CUDA.
  */

@@ -1348,23 +1348,29 @@ int ensure_teams(dp_matrix *mat, int32_t slots) {
   return DP_OK;
 }
 
-// Device staging for `count` host bound vectors, grown when needed.
-int stage_teams(TeamWs *t, int64_t count, size_t n) {
-  if (t->stage_cap >= count) return DP_OK;
-  double **bufs[4] = {&t->st_lb, &t->st_ub, &t->out_lb, &t->out_ub};
-  t->stage_cap = 0;
-  for (double **b : bufs) {
-    dp::dev_free(*b);
-    *b = nullptr;
-    void *q = nullptr;
-    const cudaError_t e = dp::dev_malloc(&q, sizeof(double) * (size_t)count * (n > 0 ? n : 1));
-    if (e != cudaSuccess) {
-      cudaGetLastError();
-      return e == cudaErrorMemoryAllocation ? DP_ERR_OOM : DP_ERR_CUDA;
+// Host bound vectors are staged kTeamStage entries at a time (more if the teams
+// that run side by side hold more): a batch of many nodes over many variables and
+// few nonzeros would need gigabytes else.
+constexpr int64_t kTeamStage = int64_t(1) << 22;
+
+// A device buffer for `count` staged bound vectors (the others' size grows with it).
+int stage_team(TeamWs *t, double **buf, int64_t count, size_t n) {
+  if (t->stage_cap < count) {
+    for (double **b : {&t->st_lb, &t->st_ub, &t->out_lb, &t->out_ub}) {
+      dp::dev_free(*b);
+      *b = nullptr;
     }
-    *b = static_cast<double *>(q);
+    t->stage_cap = count;
   }
-  t->stage_cap = count;
+  if (*buf) return DP_OK;
+  void *q = nullptr;
+  const cudaError_t e =
+      dp::dev_malloc(&q, sizeof(double) * (size_t)t->stage_cap * (n > 0 ? n : 1));
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return e == cudaErrorMemoryAllocation ? DP_ERR_OOM : DP_ERR_CUDA;
+  }
+  *buf = static_cast<double *>(q);
   return DP_OK;
 }
 
@@ -1382,7 +1388,13 @@ int nodes_by_teams(dp_ctx *ctx, dp_matrix *mat, int32_t count, const double *lb,
   TeamWs *t = mat->teams;
   const bool hl = n > 0 && !is_device_ptr(lb), hu = n > 0 && !is_device_ptr(ub);
   const bool hol = n > 0 && !is_device_ptr(lb_out), hou = n > 0 && !is_device_ptr(ub_out);
-  if ((hl || hu || hol || hou) && (rc = stage_teams(t, count, n))) return rc;
+  int32_t per = count;  // nodes of a launch
+  if (hl || hu || hol || hou)
+    per = (int32_t)std::min<int64_t>(count, std::max<int64_t>(teams, kTeamStage / (int64_t)n));
+  if (hl && (rc = stage_team(t, &t->st_lb, per, n))) return rc;
+  if (hu && (rc = stage_team(t, &t->st_ub, per, n))) return rc;
+  if (hol && (rc = stage_team(t, &t->out_lb, per, n))) return rc;
+  if (hou && (rc = stage_team(t, &t->out_ub, per, n))) return rc;
   if (t->res_cap < count) {
     if (t->h_res) cudaFreeHost(t->h_res);
     t->h_res = nullptr;
@@ -1393,28 +1405,31 @@ int nodes_by_teams(dp_ctx *ctx, dp_matrix *mat, int32_t count, const double *lb,
     }
     t->res_cap = count;
   }
-  const size_t bytes = sizeof(double) * (size_t)count * n;
   dp::TeamArgs A = t->A;
-  A.lb = lb;
-  A.ub = ub;
   A.vt = vartype;
   A.lhs = lhs;
   A.rhs = rhs;
-  if (hl) { CUDA_TRY(cudaMemcpyAsync(t->st_lb, lb, bytes, cudaMemcpyDefault, st)); A.lb = t->st_lb; }
-  if (hu) { CUDA_TRY(cudaMemcpyAsync(t->st_ub, ub, bytes, cudaMemcpyDefault, st)); A.ub = t->st_ub; }
   if (n > 0 && !is_device_ptr(vartype)) { CUDA_TRY(cudaMemcpyAsync(mat->st_vt, vartype, n, cudaMemcpyDefault, st)); A.vt = mat->st_vt; }
   if (m > 0 && !is_device_ptr(lhs)) { CUDA_TRY(cudaMemcpyAsync(mat->st_lhs, lhs, 8 * m, cudaMemcpyDefault, st)); A.lhs = mat->st_lhs; }
   if (m > 0 && !is_device_ptr(rhs)) { CUDA_TRY(cudaMemcpyAsync(mat->st_rhs, rhs, 8 * m, cudaMemcpyDefault, st)); A.rhs = mat->st_rhs; }
-  A.lb_out = hol ? t->out_lb : lb_out;
-  A.ub_out = hou ? t->out_ub : ub_out;
   A.in_stride = (int64_t)n;
-  A.res = t->h_res;
-  A.count = count;
   A.sides_ready = 1;
   team_params(A, p);
-  CUDA_TRY(dp::launch_cluster_teams(A, teams, 1 << k, ctx->num_sms, st));
-  if (hol) CUDA_TRY(cudaMemcpyAsync(lb_out, A.lb_out, bytes, cudaMemcpyDefault, st));
-  if (hou) CUDA_TRY(cudaMemcpyAsync(ub_out, A.ub_out, bytes, cudaMemcpyDefault, st));
+  for (int32_t s0 = 0; s0 < count; s0 += per) {
+    const int32_t cnt = std::min(per, count - s0);
+    const size_t off = (size_t)s0 * n, bytes = sizeof(double) * (size_t)cnt * n;
+    if (hl) CUDA_TRY(cudaMemcpyAsync(t->st_lb, lb + off, bytes, cudaMemcpyDefault, st));
+    if (hu) CUDA_TRY(cudaMemcpyAsync(t->st_ub, ub + off, bytes, cudaMemcpyDefault, st));
+    A.lb = hl ? t->st_lb : (n > 0 ? lb + off : lb);
+    A.ub = hu ? t->st_ub : (n > 0 ? ub + off : ub);
+    A.lb_out = hol ? t->out_lb : (n > 0 ? lb_out + off : lb_out);
+    A.ub_out = hou ? t->out_ub : (n > 0 ? ub_out + off : ub_out);
+    A.res = t->h_res + s0;
+    A.count = cnt;
+    CUDA_TRY(dp::launch_cluster_teams(A, std::min(teams, cnt), 1 << k, ctx->num_sms, st));
+    if (hol) CUDA_TRY(cudaMemcpyAsync(lb_out + off, t->out_lb, bytes, cudaMemcpyDefault, st));
+    if (hou) CUDA_TRY(cudaMemcpyAsync(ub_out + off, t->out_ub, bytes, cudaMemcpyDefault, st));
+  }
   CUDA_TRY(cudaStreamSynchronize(st));
   bool any_cap = false;
   for (int32_t i = 0; i < count; ++i)

@@ -1,0 +1,48 @@
+"""The rules that choose between a thread block cluster per problem (or node)
+and the graph's or batched kernels: what they bound (padding, memory, the
+number of problems, the size of a cluster), and that results are the same on
+both sides of each."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2009_07785_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+def dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+def system(lengths, n, seed, fixed=0.0):
+    rng = np.random.default_rng(seed)
+    lengths = np.asarray(lengths)
+    col = synth._distinct_columns(rng, lengths, n)
+    val = np.where(rng.random(col.size) < 0.5, -1.0, 1.0) * rng.integers(1, 11, col.size)
+    vt, lb, ub, x = synth._tiny_like_vars(rng, n)
+    rp = synth._row_ptr(lengths)
+    lhs, rhs = synth._sides(rng, rp, col, val, x, ranged_frac=0.1)
+    fix = rng.random(n) < fixed
+    lb, ub = np.where(fix, x, lb), np.where(fix, x, ub)
+    return synth.Instance("dispatch", lengths.size, n, rp, col, val, lb, ub, vt, lhs, rhs, x)
+
+
+def test_host_nodes_are_staged_in_pieces(gpu):
+    """1,200 host bound vectors of 16,000 variables, few nonzeros: 614 MB if
+    staged at once.  The results are those of device-resident vectors."""
+    dp, ctx = gpu
+    inst = system([5] * 20, 16000, seed=4)
+    LB, UB = synth.node_bounds_at_point(inst, 1200, seed=9)
+    with dp.Matrix(ctx, inst.m, inst.n, inst.row_ptr, inst.col, inst.val) as mat:
+        sides = [dev(a) for a in (inst.vartype, inst.lhs, inst.rhs)]
+        d = dp.dp_propagate_nodes(ctx, mat, dev(LB), dev(UB), *sides)
+        lb, ub = d.lb.cpu().numpy(), d.ub.cpu().numpy()
+        torch.cuda.synchronize()
+        free0 = torch.cuda.mem_get_info()[0]
+        h = dp.dp_propagate_nodes(ctx, mat, LB, UB, inst.vartype, inst.lhs, inst.rhs)
+        assert free0 - torch.cuda.mem_get_info()[0] < 300e6
+        one = dp.dp_propagate_nodes(ctx, mat, LB[1100:], dev(UB[1100:]), *sides)
+    assert np.array_equal(h.lb, lb) and np.array_equal(h.ub, ub)
+    assert np.array_equal(h.rounds, d.rounds) and np.array_equal(h.infeasible, d.infeasible)
+    assert np.array_equal(one.lb, lb[1100:]) and np.array_equal(one.rounds, d.rounds[1100:])
