@@ -116,11 +116,18 @@ constexpr int64_t kTeamNodeWork = 2500000;  // nonzeros times nodes: up to kTeam
 constexpr int64_t kTeamNodeWorkLong = 1000000;  // and above
 constexpr int kTeamWarps = 8;  // warps per block of a team
 
-// Blocks of a team, a power of two: no more than give every slice a warp and
-// all `count` teams room at once.
-int team_size(const dp_ctx *ctx, int32_t nslices, int32_t count) {
+// What the warps of a team share out in a round: the slices, the long ones
+// chunk by chunk.
+int64_t team_items(int32_t nslices, int32_t nlong) {
+  return nslices + (int64_t)(dp::kSliceW - 1) * nlong;
+}
+
+// Blocks of a team, a power of two: no more than give every item a warp and
+// all `count` teams room at once.  (With a warp per slice 100 rows of 200
+// nonzeros had one block: 691 us per call, with 16 blocks 197.)
+int team_size(const dp_ctx *ctx, int64_t items, int32_t count) {
   int k = 4;
-  while (k > 0 && ((1 << k) > 2 * ((nslices + kTeamWarps - 1) / kTeamWarps) - 1 ||
+  while (k > 0 && ((1 << k) > 2 * ((items + kTeamWarps - 1) / kTeamWarps) - 1 ||
                    ctx->teams_of[k] < count))
     --k;
   return k;  // log2
@@ -647,7 +654,8 @@ int dp_matrix_load_set(dp_ctx *ctx, int32_t count, const int32_t *m, const int32
   if (lrc) return lrc;
   const dp::TeamView &V = views.front();
   set->largest = m[V.id] > 0 ? row_ptr[V.id][m[V.id]] : 0;
-  set->view_slices = (V.split1 - V.split0) + (V.whole1 - V.whole0);
+  set->view_items =
+      team_items((V.split1 - V.split0) + (V.whole1 - V.whole0), V.nlsplit + V.nlwhole);
   *out = set;
   return DP_OK;
 }
@@ -873,7 +881,8 @@ int team_call(dp_ctx *ctx, dp_matrix *mat, const double *lb, const double *ub,
   A.res = mat->h_res;
   A.count = count;
   team_params(A, p);
-  const int k = team_size(ctx, mat->ninst > 0 ? mat->view_slices : A.M.nslices, count);
+  const int k = team_size(
+      ctx, mat->ninst > 0 ? mat->view_items : team_items(A.M.nslices, A.M.nlong), count);
   const int32_t teams = count < ctx->teams_of[k] ? count : ctx->teams_of[k];
   CUDA_TRY(dp::launch_cluster_teams(A, teams, 1 << k, ctx->num_sms, st));
   if (!dl) CUDA_TRY(cudaMemcpyAsync(lb_out, A.lb_out, 8 * n, cudaMemcpyDefault, st));
@@ -1381,7 +1390,7 @@ int nodes_by_teams(dp_ctx *ctx, dp_matrix *mat, int32_t count, const double *lb,
                    int32_t *rounds, int32_t *status) {
   const size_t n = (size_t)mat->M.n, m = (size_t)mat->M.m;
   cudaStream_t st = ctx->stream;
-  const int k = team_size(ctx, mat->M.nslices, count);
+  const int k = team_size(ctx, team_items(mat->M.nslices, mat->M.nlong), count);
   const int32_t teams = count < ctx->teams_of[k] ? count : ctx->teams_of[k];
   int rc = ensure_teams(mat, teams);
   if (rc) return rc;

@@ -48,7 +48,7 @@ struct dp_matrix {
   int32_t *h_inst = nullptr;  // pinned [3*ninst], behind h_res: infeasible, rounds, status
   dp::TeamView *d_views = nullptr;  // [ninst] the problems, largest first
   int64_t largest = 0;              // nonzeros of the largest problem
-  int32_t view_slices = 0;          // and its slices
+  int64_t view_items = 0;           // and what the warps of its team share out
   int32_t *team_next = nullptr;
 };
 

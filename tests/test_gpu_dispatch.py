@@ -2,6 +2,8 @@
 and the graph's or batched kernels: what they bound (padding, memory, the
 number of problems, the size of a cluster), and that results are the same on
 both sides of each."""
+import time
+
 import numpy as np
 import pytest
 import torch
@@ -46,3 +48,21 @@ def test_host_nodes_are_staged_in_pieces(gpu):
     assert np.array_equal(h.lb, lb) and np.array_equal(h.ub, ub)
     assert np.array_equal(h.rounds, d.rounds) and np.array_equal(h.infeasible, d.infeasible)
     assert np.array_equal(one.lb, lb[1100:]) and np.array_equal(one.rounds, d.rounds[1100:])
+
+
+def test_cluster_is_sized_by_long_chunks(gpu):
+    """100 rows of 200 nonzeros: a warp per row wants 16 blocks.  With one, as a
+    warp per 32 rows would have it, the call took 2.5 times as long as the
+    host-driven loop's kernels."""
+    dp, ctx = gpu
+    inst = system([200] * 100, 400, seed=400, fixed=0.8)
+    d = [dev(a) for a in inst.problem()]
+    with dp.Matrix(ctx, inst.m, inst.n, inst.row_ptr, inst.col, inst.val, 0, inst.lhs,
+                   inst.rhs) as mat:
+        call, loop = [], []
+        for _ in range(12):
+            t0 = time.perf_counter()
+            dp.dp_propagate(ctx, mat, *d)
+            call.append((time.perf_counter() - t0) * 1e3)
+            loop.append(sum(dp.dp_propagate_hostloop(ctx, mat, *d, timing=True).kernel_ms))
+    assert min(call) < 1.6 * min(loop), (min(call), min(loop))
