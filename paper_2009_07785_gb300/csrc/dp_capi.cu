@@ -111,6 +111,9 @@ constexpr int32_t kMarkShare = 32;
 constexpr int64_t kTeamNnz = 100000;       // a single problem, a set's largest, a node
                                            // batch's matrix without long slices
 constexpr int64_t kTeamSetNnz = 4000000;   // a whole set
+constexpr int32_t kTeamSetCount = 8192;    // its problems; three times as many
+constexpr int64_t kTeamSetFew = 1000000;   // if they have this many nonzeros or fewer
+constexpr int64_t kTeamSetPad = 24;        // its slots per nonzero
 constexpr int64_t kTeamNodeNnz = 300000;   // the matrix of a node batch with long slices
 constexpr int64_t kTeamNodeWork = 2500000;  // nonzeros times nodes: up to kTeamNnz nonzeros,
 constexpr int64_t kTeamNodeWorkLong = 1000000;  // and above
@@ -382,8 +385,8 @@ int dp_matrix_load(dp_ctx *ctx, int32_t m, int32_t n, int64_t nnz,
 namespace {
 
 // Loads a matrix from its host layout; with row_off/var_off (count+1 offsets
-// each) it is the block-diagonal union of `count` independent problems, whose
-// `views` come largest first.
+// each) it is the block-diagonal union of `count` independent problems; with
+// `views` (largest first) it was laid out problem by problem.
 int load_layout(dp_ctx *ctx, dp::HostLayout &H, const std::vector<int32_t> *row_off,
                 const std::vector<int32_t> *var_off, const std::vector<dp::TeamView> *views,
                 dp_matrix **out) {
@@ -408,28 +411,48 @@ int load_layout(dp_ctx *ctx, dp::HostLayout &H, const std::vector<int32_t> *row_
   M.mp_nseg = H.mp_nseg;
   M.mp_nlong = H.mp_nlong;
   M.mp_npiece = (int32_t)H.mp_piece.size();
-  // the order in which a round takes the slices
+  // the order in which a round takes the slices, and the candidate queues' room: the
+  // slots of their slices (merge path: the nonzeros of every 32 rows in the
+  // layout's order)
   std::vector<int32_t> order;
+  std::vector<uint32_t> qbase;
   M.short0 = H.nslices;
-  if (H.layout == dp::kLayoutEll) {
-    auto len = [&](int32_t q) { return H.slice_len[(size_t)q]; };
-    auto is_short = [&](int32_t q) { return q >= H.nslices_split && len(q) <= dp::kShortRow; };
-    for (int32_t q = 0; q < H.nslices; ++q) {
-      M.nlong += len(q) >= dp::kLongSlots;
-      M.max_slots = std::max(M.max_slots, len(q));
+  try {
+    if (H.layout == dp::kLayoutEll) {
+      auto len = [&](int32_t q) { return H.slice_len[(size_t)q]; };
+      auto is_short = [&](int32_t q) { return q >= H.nslices_split && len(q) <= dp::kShortRow; };
+      for (int32_t q = 0; q < H.nslices; ++q) {
+        M.nlong += len(q) >= dp::kLongSlots;
+        M.max_slots = std::max(M.max_slots, len(q));
+      }
+      if (views) {
+        order.resize((size_t)H.nslices);
+        for (int32_t q = 0; q < H.nslices; ++q) order[(size_t)q] = q;
+        std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) {
+          return is_short(x) != is_short(y) ? is_short(y) : len(x) > len(y);
+        });
+        while (M.short0 > 0 && is_short(order[(size_t)M.short0 - 1])) --M.short0;
+      } else {  // both kinds of slices are sorted, longest first
+        while (M.long_split < M.nslices_split && len(M.long_split) >= dp::kLongSlots) ++M.long_split;
+        M.long_whole = M.nlong - M.long_split;
+        while (M.short0 > 0 && is_short(M.short0 - 1)) --M.short0;
+      }
     }
+    std::vector<int64_t> room(dp::kQueues, 0);
+    for (int32_t q = 0; q < H.nslices; ++q)
+      for (int t = 0; t < dp::kSliceW; ++t)
+        room[(size_t)(q % dp::kQueues)] +=
+            H.chunk_len[(size_t)q * dp::kSliceW + (size_t)t] & dp::kLenMask;
+    qbase.assign(dp::kQueues, 0);
+    for (size_t q = 1; q < qbase.size(); ++q)
+      qbase[q] = (uint32_t)(qbase[q - 1] + room[q - 1]);
     if (row_off) {
-      order.resize((size_t)H.nslices);
-      for (int32_t q = 0; q < H.nslices; ++q) order[(size_t)q] = q;
-      std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) {
-        return is_short(x) != is_short(y) ? is_short(y) : len(x) > len(y);
-      });
-      while (M.short0 > 0 && is_short(order[(size_t)M.short0 - 1])) --M.short0;
-    } else {  // both kinds of slices are sorted, longest first
-      while (M.long_split < M.nslices_split && len(M.long_split) >= dp::kLongSlots) ++M.long_split;
-      M.long_whole = M.nlong - M.long_split;
-      while (M.short0 > 0 && is_short(M.short0 - 1)) --M.short0;
+      mat->row_off = *row_off;
+      mat->var_off = *var_off;
     }
+  } catch (const std::bad_alloc &) {
+    dp_matrix_free(mat);
+    return DP_ERR_OOM;
   }
   mat->padded = (int64_t)H.val.size();
 #define TRY(x)                 \
@@ -476,18 +499,6 @@ int load_layout(dp_ctx *ctx, dp::HostLayout &H, const std::vector<int32_t> *row_
   // candidate queue: at most one entry per slot and round, so it never
   // overflows; row sums are stored per chunk slot
   TRY(dev_alloc(mat, &S.queue, (size_t)mat->padded));
-  // the queues' room: the slots of their slices (merge path: the nonzeros of
-  // every 32 rows in the layout's order)
-  std::vector<uint32_t> qbase(dp::kQueues, 0);
-  {
-    std::vector<int64_t> room(dp::kQueues, 0);
-    for (int32_t q = 0; q < H.nslices; ++q)
-      for (int t = 0; t < dp::kSliceW; ++t)
-        room[(size_t)(q % dp::kQueues)] +=
-            H.chunk_len[(size_t)q * dp::kSliceW + (size_t)t] & dp::kLenMask;
-    for (size_t q = 1; q < qbase.size(); ++q)
-      qbase[q] = (uint32_t)(qbase[q - 1] + room[q - 1]);
-  }
   TRY(upload(mat, qbase, &S.qbase, st));
   TRY(dev_alloc(mat, &S.qcount, (size_t)dp::kQueues * dp::kQueueStep));
   if (cudaMemsetAsync(S.qcount, 0, sizeof(int32_t) * dp::kQueues * dp::kQueueStep, st) !=
@@ -553,12 +564,12 @@ int load_layout(dp_ctx *ctx, dp::HostLayout &H, const std::vector<int32_t> *row_
     TRY(dev_alloc(mat, &S.I.status, (size_t)count));
     S.I.ninst = count;
     mat->ninst = count;
-    const dp::TeamView *dv = nullptr;
-    TRY(upload(mat, *views, &dv, st));
-    mat->d_views = const_cast<dp::TeamView *>(dv);
-    TRY(dev_alloc(mat, &mat->team_next, 1));
-    mat->row_off = *row_off;
-    mat->var_off = *var_off;
+    if (views) {
+      const dp::TeamView *dv = nullptr;
+      TRY(upload(mat, *views, &dv, st));
+      mat->d_views = const_cast<dp::TeamView *>(dv);
+      TRY(dev_alloc(mat, &mat->team_next, 1));
+    }
     int4 *pinned = nullptr;
     if (cudaMallocHost(&pinned, (sizeof(int4) + 3 * sizeof(int32_t)) * (size_t)count) !=
         cudaSuccess) {
@@ -596,6 +607,69 @@ int load_impl(dp_ctx *ctx, int32_t m, int32_t n, int64_t nnz, const int64_t *row
   return load_layout(ctx, H, nullptr, nullptr, nullptr, out);
 }
 
+// Whether a set is loaded problem by problem, for a team each, and not as one
+// union whose rows share length-sorted slices: small problems, not too many of
+// them, and no more than kTeamSetPad slots to a nonzero (every problem is padded
+// to whole slices, up to 32 slots to a nonzero for problems of one row).
+bool set_by_teams(const dp_ctx *ctx, int32_t count, const int32_t *m,
+                  const int64_t *const *row_ptr, int64_t nnz, int32_t chunk) {
+  if (ctx->teams_of[0] <= 0 || nnz > kTeamSetNnz ||
+      count > (nnz <= kTeamSetFew ? 3 : 1) * kTeamSetCount)
+    return false;
+  if (chunk == 0) chunk = 256;
+  if (chunk < 8) return false;  // refused by the layout
+  int64_t slots = 0;
+  std::vector<int32_t> whole, piece;
+  for (int32_t k = 0; k < count; ++k) {
+    whole.clear();
+    piece.clear();
+    if (m[k] > 0 && row_ptr[k][m[k]] > kTeamNnz) return false;
+    for (int32_t i = 0; i < m[k]; ++i) {
+      int64_t len = row_ptr[k][i + 1] - row_ptr[k][i];
+      if (len < 0 || len > nnz) return false;  // refused by the layout
+      if (len <= chunk) {
+        whole.push_back((int32_t)len);
+        continue;
+      }
+      for (; len > 0; len -= chunk) piece.push_back((int32_t)(len < chunk ? len : chunk));
+    }
+    for (std::vector<int32_t> *v : {&whole, &piece}) {
+      std::sort(v->begin(), v->end(), [](int32_t x, int32_t y) { return x > y; });
+      for (size_t q = 0; q < v->size(); q += dp::kSliceW) slots += (int64_t)dp::kSliceW * (*v)[q];
+    }
+  }
+  return slots <= kTeamSetPad * nnz;
+}
+
+// The layout of the block-diagonal union as one matrix.
+int build_union(int32_t count, const int32_t *m, const int32_t *n, const int64_t *const *row_ptr,
+                const int32_t *const *col_idx, const double *const *val, int32_t chunk,
+                const double *const *lhs, const double *const *rhs, int32_t rows, int64_t nnz,
+                const std::vector<int32_t> &var_off, dp::HostLayout &H) {
+  std::vector<int64_t> rp(1, 0);
+  std::vector<int32_t> col;
+  std::vector<double> vv, sl, sr;
+  rp.reserve((size_t)rows + 1);
+  col.reserve((size_t)std::max<int64_t>(nnz, 0));
+  vv.reserve((size_t)std::max<int64_t>(nnz, 0));
+  for (int32_t k = 0; k < count; ++k) {
+    const int64_t base = rp.back(), nz = m[k] > 0 ? row_ptr[k][m[k]] : 0;
+    for (int32_t i = 0; i < m[k]; ++i) rp.push_back(base + row_ptr[k][i + 1]);
+    for (int64_t q = 0; q < nz; ++q) {
+      const int32_t c = col_idx[k][q];
+      if (c < 0 || c >= n[k]) return DP_ERR_BAD_CSR;
+      col.push_back(c + var_off[(size_t)k]);
+      vv.push_back(val[k][q]);
+    }
+    if (lhs) {
+      sl.insert(sl.end(), lhs[k], lhs[k] + m[k]);
+      sr.insert(sr.end(), rhs[k], rhs[k] + m[k]);
+    }
+  }
+  return dp::build_layout(rows, var_off.back(), nnz, rp.data(), col.data(), vv.data(), chunk,
+                          lhs ? sl.data() : nullptr, lhs ? sr.data() : nullptr, H);
+}
+
 }  // namespace
 
 extern "C" {
@@ -629,35 +703,45 @@ int dp_matrix_load_set(dp_ctx *ctx, int32_t count, const int32_t *m, const int32
     return DP_ERR_INVALID_ARG;
   *out = nullptr;
   if ((lhs == nullptr) != (rhs == nullptr)) return DP_ERR_INVALID_ARG;
-  std::vector<int32_t> row_off(1, 0), var_off(1, 0);
-  int64_t mt = 0, nt = 0, nzt = 0;
-  for (int32_t k = 0; k < count; ++k) {
-    if (m[k] < 0 || n[k] < 0 || (m[k] > 0 && !row_ptr[k])) return DP_ERR_INVALID_ARG;
-    mt += m[k];
-    nt += n[k];
-    if (m[k] > 0) nzt += row_ptr[k][m[k]];
-    if (mt >= (int64_t(1) << 31) || nt >= (int64_t(1) << 31) || nzt >= (int64_t(1) << 31))
-      return DP_ERR_INVALID_ARG;
-    row_off.push_back((int32_t)mt);
-    var_off.push_back((int32_t)nt);
+  try {
+    std::vector<int32_t> row_off(1, 0), var_off(1, 0);
+    int64_t mt = 0, nt = 0, nzt = 0;
+    for (int32_t k = 0; k < count; ++k) {
+      if (m[k] < 0 || n[k] < 0 || (m[k] > 0 && !row_ptr[k])) return DP_ERR_INVALID_ARG;
+      mt += m[k];
+      nt += n[k];
+      if (m[k] > 0) nzt += row_ptr[k][m[k]];
+      if (mt >= (int64_t(1) << 31) || nt >= (int64_t(1) << 31) || nzt >= (int64_t(1) << 31))
+        return DP_ERR_INVALID_ARG;
+      row_off.push_back((int32_t)mt);
+      var_off.push_back((int32_t)nt);
+    }
+    for (int32_t k = 0; k < count; ++k) {
+      if (m[k] > 0 && row_ptr[k][0] != 0) return DP_ERR_BAD_CSR;
+      if (m[k] > 0 && row_ptr[k][m[k]] > 0 && (!col_idx[k] || !val[k])) return DP_ERR_INVALID_ARG;
+    }
+    dp::HostLayout H;
+    std::vector<dp::TeamView> views;
+    int rc;
+    if (set_by_teams(ctx, count, m, row_ptr, nzt, chunk))
+      rc = dp::build_set_layout(count, m, n, row_ptr, col_idx, val, chunk, lhs, rhs, H, views);
+    else
+      rc = build_union(count, m, n, row_ptr, col_idx, val, chunk, lhs, rhs, (int32_t)mt, nzt,
+                       var_off, H);
+    if (rc) return rc;
+    dp_matrix *set = nullptr;
+    rc = load_layout(ctx, H, &row_off, &var_off, views.empty() ? nullptr : &views, &set);
+    if (rc) return rc;
+    if (!views.empty()) {
+      const dp::TeamView &V = views.front();
+      set->view_items =
+          team_items((V.split1 - V.split0) + (V.whole1 - V.whole0), V.nlsplit + V.nlwhole);
+    }
+    *out = set;
+    return DP_OK;
+  } catch (const std::bad_alloc &) {
+    return DP_ERR_OOM;
   }
-  for (int32_t k = 0; k < count; ++k) {
-    if (m[k] > 0 && row_ptr[k][0] != 0) return DP_ERR_BAD_CSR;
-    if (m[k] > 0 && row_ptr[k][m[k]] > 0 && (!col_idx[k] || !val[k])) return DP_ERR_INVALID_ARG;
-  }
-  dp::HostLayout H;
-  std::vector<dp::TeamView> views;
-  const int rc = dp::build_set_layout(count, m, n, row_ptr, col_idx, val, chunk, lhs, rhs, H, views);
-  if (rc) return rc;
-  dp_matrix *set = nullptr;
-  const int lrc = load_layout(ctx, H, &row_off, &var_off, &views, &set);
-  if (lrc) return lrc;
-  const dp::TeamView &V = views.front();
-  set->largest = m[V.id] > 0 ? row_ptr[V.id][m[V.id]] : 0;
-  set->view_items =
-      team_items((V.split1 - V.split0) + (V.whole1 - V.whole0), V.nlsplit + V.nlwhole);
-  *out = set;
-  return DP_OK;
 }
 
 int dp_matrix_set_launch(dp_matrix *mat, int32_t round_warps) {
@@ -841,11 +925,6 @@ int check_call(dp_ctx *ctx, const dp_matrix *mat, const double *lb, const double
   return DP_OK;
 }
 
-// Whether teams, one per problem, beat the graph over the union.
-bool teams_for_set(const dp_matrix *set) {
-  return set->h_res && set->largest <= kTeamNnz && set->M.nnz <= kTeamSetNnz;
-}
-
 // The whole propagation of one small problem by one team, or of every problem
 // of a set by a team each; results in mat->h_res.
 int team_call(dp_ctx *ctx, dp_matrix *mat, const double *lb, const double *ub,
@@ -968,7 +1047,7 @@ int set_call(dp_ctx *ctx, const dp_matrix *cset, const double *lb, const double 
       return DP_ERR_CUDA;
   }
   dp_matrix *set = const_cast<dp_matrix *>(cset);
-  if (!persistent && !set->M.val8 && ctx->teams_of[0] > 0 && teams_for_set(set)) {
+  if (!persistent && !set->M.val8 && set->d_views) {  // loaded for a team per problem
     rc = team_call(ctx, set, lb, ub, vartype, lhs, rhs, p, lb_out, ub_out);
     if (rc < 0) return rc;
     bool cap = false;

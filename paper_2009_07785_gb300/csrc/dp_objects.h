@@ -46,9 +46,8 @@ struct dp_matrix {
   int32_t ninst = 0;
   std::vector<int32_t> row_off, var_off;
   int32_t *h_inst = nullptr;  // pinned [3*ninst], behind h_res: infeasible, rounds, status
-  dp::TeamView *d_views = nullptr;  // [ninst] the problems, largest first
-  int64_t largest = 0;              // nonzeros of the largest problem
-  int64_t view_items = 0;           // and what the warps of its team share out
+  dp::TeamView *d_views = nullptr;  // [ninst] the problems, largest first (null: one union)
+  int64_t view_items = 0;           // what the warps of the largest one's team share out
   int32_t *team_next = nullptr;
 };
 

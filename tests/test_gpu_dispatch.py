@@ -9,6 +9,7 @@ import pytest
 import torch
 
 from paper_2009_07785_gb300 import synth
+from parity import compare_bounds
 
 pytestmark = pytest.mark.gpu
 
@@ -28,6 +29,51 @@ def system(lengths, n, seed, fixed=0.0):
     fix = rng.random(n) < fixed
     lb, ub = np.where(fix, x, lb), np.where(fix, x, ub)
     return synth.Instance("dispatch", lengths.size, n, rp, col, val, lb, ub, vt, lhs, rhs, x)
+
+
+def check_set(dp, ctx, orc, ps, sample, slots_per_nnz):
+    arrays = [dev(np.concatenate([getattr(p, a) for p in ps]))
+              for a in ("lb", "ub", "vartype", "lhs", "rhs")]
+    with dp.MatrixSet(ctx, ps, 0, sides=True) as ms:
+        info, off = ms.info(), ms.var_off
+        r = dp.dp_propagate_set(ctx, ms, *arrays)
+        q = dp.dp_propagate_set_persistent(ctx, ms, *arrays)
+    assert info["padded_slots"] <= slots_per_nnz * info["nnz"]
+    assert np.array_equal(r.rounds, q.rounds) and np.array_equal(r.infeasible, q.infeasible)
+    assert torch.equal(r.lb, q.lb) and torch.equal(r.ub, q.ub)
+    for k in sample:
+        p = ps[k]
+        o = orc.propagate_instance(p)
+        assert o.rounds == r.rounds[k] and o.infeasible == r.infeasible[k], k
+        s = slice(off[k], off[k + 1])
+        nbad, _, det = compare_bounds(r.lb[s].cpu().numpy(), r.ub[s].cpu().numpy(), o.lb, o.ub,
+                                      p.vartype)
+        assert nbad == 0, det
+
+
+def test_set_of_one_row_problems_shares_slices(gpu, orc):
+    """Laid out problem by problem, a row alone in its slice would take 32 slots
+    to a nonzero."""
+    dp, ctx = gpu
+    ps = [system([40 + k % 7], 64, seed=k) for k in range(3000)]
+    check_set(dp, ctx, orc, ps, range(0, 3000, 301), slots_per_nnz=1.1)
+
+
+def test_set_of_many_problems_shares_slices(gpu, orc):
+    """More problems than clusters run well one after the other."""
+    dp, ctx = gpu
+    some = [synth.tiny(seed=k, m=20, n=16) for k in range(300)]
+    check_set(dp, ctx, orc, [some[k % 300] for k in range(9000)], range(0, 9000, 901),
+              slots_per_nnz=1.1)
+
+
+@pytest.mark.parametrize("counts", [(2, 3, 1), (24, 2)])
+def test_set_of_few_rows_each(gpu, orc, counts):
+    """Sets on the padded side of the rule: few slots, a cluster each."""
+    dp, ctx = gpu
+    rows, times = counts[:-1], counts[-1]
+    ps = [synth.tiny(seed=k, m=m, n=16) for k in range(40 * times) for m in rows]
+    check_set(dp, ctx, orc, ps, range(0, len(ps), 9), slots_per_nnz=24)
 
 
 def test_host_nodes_are_staged_in_pieces(gpu):
