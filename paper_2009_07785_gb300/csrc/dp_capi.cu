@@ -94,22 +94,29 @@ constexpr int32_t kMarkShare = 32;
 // Where a team (dp_team.cu) takes a problem instead of the graph's kernels or
 // the batched ones.  A team's rounds cost less (a cluster barrier instead of
 // three to five kernels) and its marking skips unchanged rows, but it has 16
-// blocks at most.  Measured in us per call (graph or batch / team):
-//   one problem:  short rows 60k nonzeros 460 / 384, 179k 571 / 797;
-//                 irregular 60k 1112 / 634, 235k 1397 / 1275, 704k 2211 / 3790;
-//                 mixed 25k 1796 / 866, 126k 1750 / 1327, 378k 2187 / 2748
-//   nodes:        irregular 60k nonzeros, 8 nodes 1296 / 705, 33 nodes
-//                 1560 / 1077, 100 nodes 1831 / 1825; 187k, 8 nodes 1694 / 1310
-//                 in many rounds but 188 / 233 in one, 16 nodes 1715 / 1991;
-//                 235k, 1 node 2445 / 1264 and 175 / 213;
-//                 short rows 60k, 8 nodes 678 / 456, 33 nodes 956 / 706,
-//                 100 nodes 1373 / 1707; 239k, 1 node 793 / 961, 16 nodes
-//                 1097 / 1639: without long chunks, which a team spreads over
-//                 its warps, the team's few blocks bound it sooner
-//   sets:         12 problems of up to 29k nonzeros 2855 / 842; 64 of up to
-//                 1.7M 8331 / 22885
+// blocks at most.  Measured in us per call (graph or batch / team), both in one
+// run of the same build:
+//   one problem:  short rows 50k nonzeros 542 / 405, 100k 605 / 582, 140k 533 / 681;
+//                 irregular 55k 832 / 749, 110k 853 / 781, 226k 1187 / 1318;
+//                 mixed 42k 1185 / 865, 80k 1036 / 1068, 116k 1375 / 1620;
+//                 90k in rows of 3 (938 slices) 346 / 458, of 6 (470) 510 / 497
+//   nodes:        irregular 60k nonzeros, 8 nodes 1521 / 772 in many rounds and 171 /
+//                 127 in one, 33 nodes 2221 / 1151 and 190 / 199, 100 nodes
+//                 2621 / 2166; 90k, 33 nodes 7981 / 2256 and 210 / 236; 140k, 8
+//                 nodes 3235 / 1269 and 171 / 204; 250k, 1 node 2928 / 1573 and 175 /
+//                 226, 16 nodes 3267 / 2933;
+//                 short rows 60k, 8 nodes 734 / 472, 33 nodes 953 / 672, 100 nodes
+//                 1369 / 1622; 140k, 8 nodes 823 / 725, 16 nodes 908 / 1094;
+//                 1000 nodes over 2k in rows of 6 1545 / 927 (10 items), of 30 387 /
+//                 712 (65 items); over 12k in rows of 6 2274 / 2837 (63 items)
+//   sets:         64 problems of 300 rows 770 / 352, 64 of up to 60,000 2727 / 6348;
+//                 1000 of 300 1961 / 1248; 8000 of 20 3892 / 3857, of 100 4967 /
+//                 4803; 10,000 of 20 4229 / 4738, 20,000 of 20 6701 / 8761, of 10
+//                 5696 / 5474, of 2 3255 / 2134; 50,000 of 2 3481 / 4405, 100,000 of 1
+//                 1247 / 6621
 constexpr int64_t kTeamNnz = 100000;       // a single problem, a set's largest, a node
                                            // batch's matrix without long slices
+constexpr int32_t kTeamSlices = 640;       // slices of a single problem
 constexpr int64_t kTeamSetNnz = 4000000;   // a whole set
 constexpr int32_t kTeamSetCount = 8192;    // its problems; three times as many
 constexpr int64_t kTeamSetFew = 1000000;   // if they have this many nonzeros or fewer
@@ -117,6 +124,7 @@ constexpr int64_t kTeamSetPad = 24;        // its slots per nonzero
 constexpr int64_t kTeamNodeNnz = 300000;   // the matrix of a node batch with long slices
 constexpr int64_t kTeamNodeWork = 2500000;  // nonzeros times nodes: up to kTeamNnz nonzeros,
 constexpr int64_t kTeamNodeWorkLong = 1000000;  // and above
+constexpr int64_t kTeamNodeItems = 40;     // team_items of a matrix with more nodes than teams
 constexpr int kTeamWarps = 8;  // warps per block of a team
 
 // What the warps of a team share out in a round: the slices, the long ones
@@ -987,7 +995,7 @@ int dp_propagate(dp_ctx *ctx, const dp_matrix *cmat, const double *lb,
   if (rc) return rc;
   dp_matrix *mat = const_cast<dp_matrix *>(cmat);
   if (mat->h_res && mat->ninst == 0 && !mat->M.val8 && mat->M.nnz <= kTeamNnz &&
-      ctx->teams_of[0] > 0) {
+      mat->M.nslices <= kTeamSlices && ctx->teams_of[0] > 0) {
     rc = team_call(ctx, mat, lb, ub, vartype, lhs, rhs, p, lb_out, ub_out);
     if (rc) return rc;
     *infeasible = mat->h_res->x;
@@ -1536,6 +1544,9 @@ int nodes_by_teams(dp_ctx *ctx, dp_matrix *mat, int32_t count, const double *lb,
 bool teams_for_nodes(const dp_ctx *ctx, const dp_matrix *mat, int32_t count) {
   if (!mat->h_res || ctx->teams_of[0] <= 0) return false;
   const int64_t nnz = mat->M.nnz, work = nnz * (int64_t)count;
+  // teams of one block take the nodes in several turns
+  if (count > ctx->teams_of[0] && team_items(mat->M.nslices, mat->M.nlong) > kTeamNodeItems)
+    return false;
   if (nnz <= kTeamNnz) return work <= kTeamNodeWork;
   return mat->M.nlong > 0 && nnz <= kTeamNodeNnz && work <= kTeamNodeWorkLong;
 }

@@ -96,6 +96,37 @@ def test_host_nodes_are_staged_in_pieces(gpu):
     assert np.array_equal(one.lb, lb[1100:]) and np.array_equal(one.rounds, d.rounds[1100:])
 
 
+@pytest.mark.parametrize("lengths,count", [([5] * 64, 700), ([30, 34] * 33, 700), ([30, 34] * 33, 33)])
+def test_more_nodes_than_clusters(gpu, lengths, count):
+    dp, ctx = gpu
+    inst = system(lengths, 96, seed=count)
+    LB, UB = synth.node_bounds_at_point(inst, count, seed=2)
+    args = [dev(a) for a in (LB, UB, inst.vartype, inst.lhs, inst.rhs)]
+    with dp.Matrix(ctx, inst.m, inst.n, inst.row_ptr, inst.col, inst.val) as mat:
+        a = dp.dp_propagate_nodes(ctx, mat, *args)
+        b = dp.dp_propagate_nodes_persistent(ctx, mat, *args)
+    assert np.array_equal(a.rounds, b.rounds) and np.array_equal(a.infeasible, b.infeasible)
+    assert torch.equal(a.lb, b.lb) and torch.equal(a.ub, b.ub)
+
+
+@pytest.mark.parametrize("lengths,n", [([200] * 100, 400), ([3] * 30000, 22500)])
+def test_single_problems_by_either_path(gpu, orc, lengths, n):
+    """Few long rows (a large cluster) and more slices than a cluster takes."""
+    dp, ctx = gpu
+    inst = system(lengths, n, seed=n, fixed=0.8 if lengths[0] > 100 else 0.0)
+    assert inst.nnz <= 100_000
+    d = [dev(a) for a in inst.problem()]
+    with dp.Matrix(ctx, inst.m, inst.n, inst.row_ptr, inst.col, inst.val, 0, inst.lhs,
+                   inst.rhs) as mat:
+        a = dp.dp_propagate(ctx, mat, *d)
+        b = dp.dp_propagate_hostloop(ctx, mat, *d)
+    o = orc.propagate_instance(inst)
+    assert a.rounds == b.rounds == o.rounds and a.infeasible == o.infeasible
+    assert torch.equal(a.lb, b.lb) and torch.equal(a.ub, b.ub)
+    nbad, _, det = compare_bounds(a.lb.cpu().numpy(), a.ub.cpu().numpy(), o.lb, o.ub, inst.vartype)
+    assert nbad == 0, det
+
+
 def test_cluster_is_sized_by_long_chunks(gpu):
     """100 rows of 200 nonzeros: a warp per row wants 16 blocks.  With one, as a
     warp per 32 rows would have it, the call took 2.5 times as long as the
