@@ -108,7 +108,8 @@ constexpr int32_t kMarkShare = 32;
 //                 short rows 60k, 8 nodes 734 / 472, 33 nodes 953 / 672, 100 nodes
 //                 1369 / 1622; 140k, 8 nodes 823 / 725, 16 nodes 908 / 1094;
 //                 1000 nodes over 2k in rows of 6 1545 / 927 (10 items), of 30 387 /
-//                 712 (65 items); over 12k in rows of 6 2274 / 2837 (63 items)
+//                 712 (34 items); over 4k in rows of 4 2372 / 1824 (31 items), over 12k in
+//                 rows of 6 2274 / 2837 (63 items)
 //   sets:         64 problems of 300 rows 770 / 352, 64 of up to 60,000 2727 / 6348;
 //                 1000 of 300 1961 / 1248; 8000 of 20 3892 / 3857, of 100 4967 /
 //                 4803; 10,000 of 20 4229 / 4738, 20,000 of 20 6701 / 8761, of 10
@@ -124,7 +125,7 @@ constexpr int64_t kTeamSetPad = 24;        // its slots per nonzero
 constexpr int64_t kTeamNodeNnz = 300000;   // the matrix of a node batch with long slices
 constexpr int64_t kTeamNodeWork = 2500000;  // nonzeros times nodes: up to kTeamNnz nonzeros,
 constexpr int64_t kTeamNodeWorkLong = 1000000;  // and above
-constexpr int64_t kTeamNodeItems = 40;     // team_items of a matrix with more nodes than teams
+constexpr int64_t kTeamNodeItems = 32;     // team_items of a matrix with more nodes than teams
 constexpr int kTeamWarps = 8;  // warps per block of a team
 
 // What the warps of a team share out in a round: the slices, the long ones
