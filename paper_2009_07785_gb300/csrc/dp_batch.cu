@@ -55,18 +55,18 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kActWarps = 8;
-// k_bact's work items (chunks of one node group) are handed out by ticket, the
-// split rows' first: with a fixed share per warp the warps with the longest
+// k_bact<false>'s work items (chunks of one node group) are handed out by ticket,
+// the split rows' first: with a fixed share per warp the warps with the longest
 // chunks end last, and the split rows' chunks, appended last, ended every
 // round (2.0M nonzeros, 256 nodes: random fixings 4.66 -> 4.29 ms of k_bact,
 // fixings at a point 36.4 -> 30.2).  Two items to a ticket where every warp has
 // at least 32 of them, else one: the tickets come from one counter (0.8M of
 // them in a dense round; one item each 5.5 ms, four 4.3 but 34.1 at a point).
-// Fixed shares remain below 8 items per warp if no chunk has 64 nonzeros: they
-// are even there, and a ticket costs 1.2 ns on the counter (200 nodes over 30k
-// nonzeros in short rows 660 us per call, 680 with tickets).
+// Fixed shares remain for rounds below 8 items per warp if no chunk has
+// kTicketSlots nonzeros: they are even there, and a ticket costs 1.2 ns on the
+// counter.
 constexpr int kActItems = 2;
-constexpr int kTicketItems = 8, kTicketSlots = 64;
+constexpr int kTicketItems = 8;
 
 struct BParams {
   int32_t Bp, G, Gs, round, max_rounds, err;
@@ -508,7 +508,9 @@ __device__ __forceinline__ void bmark_body(const DevMatrix &M, const BatchState 
 }
 
 // All chunks of a split row get the OR of their masks (the row's activity
-// needs every chunk), and become work items.  Block per split row.
+// needs every chunk), and become work items.  Block per split row.  kOne: behind the
+// whole rows' in one list.
+template <bool kOne>
 __device__ __forceinline__ void bmark_split_body(const DevMatrix &M, const BatchState &S) {
   BCtrl *ctrl = S.ctrl;
   const BParams P = load_params(ctrl);
@@ -547,8 +549,12 @@ __device__ __forceinline__ void bmark_split_body(const DevMatrix &M, const Batch
         if (g >= P.G || word4(m, u) == 0u) continue;  // block-uniform
         for (int32_t qb = q0 + warp * 32; qb < q1; qb += kThreads) {  // warp-uniform
           const int32_t q = qb + lane;
-          warp_append<int32_t, -1>(q < q1, q < q1 ? M.split_cidx[q] : 0,
-                                   S.items + (int64_t)(g + 1) * nslots - 1, &ctrl->scount[g]);
+          const int32_t cs = q < q1 ? M.split_cidx[q] : 0;
+          if (kOne)
+            warp_append<int32_t>(q < q1, cs, S.items + (int64_t)g * nslots, &ctrl->icount[g]);
+          else
+            warp_append<int32_t, -1>(q < q1, cs, S.items + (int64_t)(g + 1) * nslots - 1,
+                                     &ctrl->scount[g]);
         }
       }
     }
@@ -562,7 +568,8 @@ __device__ __forceinline__ int32_t item_of(const BatchState &S, int g, int q, in
   return S.items[q < scnt ? (g + 1) * S.nslots - 1 - q : g * S.nslots + (q - scnt)];
 }
 
-template <bool kCo>
+// kFixed: fixed shares of one list.
+template <bool kCo, bool kFixed = false>
 __device__ __forceinline__ void bact_body(const DevMatrix &M, const BatchState &S,
                                           PairBuf *s_pairs) {
   BCtrl *ctrl = S.ctrl;
@@ -571,7 +578,7 @@ __device__ __forceinline__ void bact_body(const DevMatrix &M, const BatchState &
   const int p = P.round & 1;
   const int lane = threadIdx.x & 31;
   // regions of the work list: lane g holds the item counts of group g
-  const int scnt = lane < P.G ? ctrl->scount[lane] : 0;
+  const int scnt = !kFixed && lane < P.G ? ctrl->scount[lane] : 0;
   const int cnt = lane < P.G ? ctrl->icount[lane] + scnt : 0;
   int incl = cnt;
 #pragma unroll
@@ -585,57 +592,64 @@ __device__ __forceinline__ void bact_body(const DevMatrix &M, const BatchState &
   const int nw = gridDim.x * kActWarps;
   PairQueue pq{&s_pairs[threadIdx.x >> 5], 0};
   uint32_t *chg_next = S.chg[p ^ 1];
-  const int bs = max(1, min(kActItems, total / (16 * nw)));
-  const int nb = (total + bs - 1) / bs;
-  // tickets only where shares can be uneven: many items, or long chunks
-  const bool tickets = nb > kTicketItems * nw || (nb > nw && M.max_slots >= kTicketSlots);
-  int next = blockIdx.x * kActWarps + (threadIdx.x >> 5);
-  while (next < nb) {
-    int it = next * bs;
-    const int end = min(total, it + bs);
-    if (!tickets) next += nw;
-    else if (lane == 0) next = nw + (int)atomicAdd(&ctrl->ticket, 1u);
-    for (; it < end; ++it) {
-      const int g = __popc(__ballot_sync(kFull, lane < P.G && it >= incl));
-      const int64_t cs = item_of(S, g, it - __shfl_sync(kFull, excl, g),
-                                 __shfl_sync(kFull, scnt, g));
-      const int node = g * 32 + lane;
-      const uint32_t mask = S.cmask[cs * P.Gs + g];
-      const bool on = ((mask >> lane) & 1u) != 0u;
-      const int32_t row = M.chunk_row[cs];
-      const int32_t lenf = M.chunk_len[cs];
-      const int len = lenf & kLenMask;
-      const bool exact = (lenf & kExactFlag) != 0;
-      const int64_t base = M.slice_off[cs / kSliceW] + (cs % kSliceW);
-      const double lhs = S.lhs[row], rhs = S.rhs[row];
-      const bool need_min = d_isfinite(rhs), need_max = d_isfinite(lhs);
-      const BAct r = chunk_activity<kCo>(M, S, base, len, node, need_min, need_max, !exact, P);
-      if (cs < split_slots) {
-        BPartial pt;
-        pt.minfin = r.minfin;
-        pt.maxfin = r.maxfin;
-        pt.mininf = r.mininf;
-        pt.maxinf = r.maxinf;
-        pt.tr = r.tr;
-        pt.tl = r.tl;
-        S.part[cs * P.Bp + node] = pt;
-        continue;
-      }
-      RowView rv;
-      rv.minfin = r.minfin;
-      rv.maxfin = r.maxfin;
-      rv.lhs = lhs;
-      rv.rhs = rhs;
-      rv.mininf = r.mininf;
-      rv.maxinf = r.maxinf;
-      rv.exact = exact ? 1 : 0;
-      const bool infeas = row_sides_eval(rv, r.tr, r.tl, P.eps_feas);
-      note_nodes(S.inf_bits, g, __ballot_sync(kFull, on && infeas));
-      const bool go = on && rv.act != 0;
-      if (!__any_sync(kFull, go)) continue;
-      chunk_candidates<kCo>(M, S, base, len, node, go, row, rv, P, pq, chg_next);
+  auto item = [&](int it) {
+    const int g = __popc(__ballot_sync(kFull, lane < P.G && it >= incl));
+    const int q = it - __shfl_sync(kFull, excl, g);
+    const int64_t cs = kFixed ? S.items[(int64_t)g * S.nslots + q]
+                              : item_of(S, g, q, __shfl_sync(kFull, scnt, g));
+    const int node = g * 32 + lane;
+    const uint32_t mask = S.cmask[cs * P.Gs + g];
+    const bool on = ((mask >> lane) & 1u) != 0u;
+    const int32_t row = M.chunk_row[cs];
+    const int32_t lenf = M.chunk_len[cs];
+    const int len = lenf & kLenMask;
+    const bool exact = (lenf & kExactFlag) != 0;
+    const int64_t base = M.slice_off[cs / kSliceW] + (cs % kSliceW);
+    const double lhs = S.lhs[row], rhs = S.rhs[row];
+    const bool need_min = d_isfinite(rhs), need_max = d_isfinite(lhs);
+    const BAct r = chunk_activity<kCo>(M, S, base, len, node, need_min, need_max, !exact, P);
+    if (cs < split_slots) {
+      BPartial pt;
+      pt.minfin = r.minfin;
+      pt.maxfin = r.maxfin;
+      pt.mininf = r.mininf;
+      pt.maxinf = r.maxinf;
+      pt.tr = r.tr;
+      pt.tl = r.tl;
+      S.part[cs * P.Bp + node] = pt;
+      return;
     }
-    next = __shfl_sync(kFull, next, 0);
+    RowView rv;
+    rv.minfin = r.minfin;
+    rv.maxfin = r.maxfin;
+    rv.lhs = lhs;
+    rv.rhs = rhs;
+    rv.mininf = r.mininf;
+    rv.maxinf = r.maxinf;
+    rv.exact = exact ? 1 : 0;
+    const bool infeas = row_sides_eval(rv, r.tr, r.tl, P.eps_feas);
+    note_nodes(S.inf_bits, g, __ballot_sync(kFull, on && infeas));
+    const bool go = on && rv.act != 0;
+    if (!__any_sync(kFull, go)) return;
+    chunk_candidates<kCo>(M, S, base, len, node, go, row, rv, P, pq, chg_next);
+  };
+  const int first = blockIdx.x * kActWarps + (threadIdx.x >> 5);
+  if constexpr (kFixed) {
+    for (int it = first; it < total; it += nw) item(it);
+  } else {
+    const int bs = max(1, min(kActItems, total / (16 * nw)));
+    const int nb = (total + bs - 1) / bs;
+    // tickets only where shares can be uneven: many items, or long chunks
+    const bool tickets = nb > kTicketItems * nw || (nb > nw && M.max_slots >= kTicketSlots);
+    int next = first;
+    while (next < nb) {
+      int it = next * bs;
+      const int end = min(total, it + bs);
+      if (!tickets) next += nw;
+      else if (lane == 0) next = nw + (int)atomicAdd(&ctrl->ticket, 1u);
+      for (; it < end; ++it) item(it);
+      next = __shfl_sync(kFull, next, 0);
+    }
   }
   drain_pairs<kCo>(pq, M, S, P, chg_next);
 }
@@ -1009,16 +1023,18 @@ __global__ void __launch_bounds__(kThreads) k_bmark(DevMatrix M, BatchState S) {
   bmark_body(M, S);
 }
 
+template <bool kOne>
 __global__ void __launch_bounds__(kThreads) k_bmark_split(DevMatrix M, BatchState S) {
-  bmark_split_body(M, S);
+  bmark_split_body<kOne>(M, S);
 }
 
 // Four blocks of eight warps per SM (64 registers, a few spilled): the
 // kernel waits on gathers, and 32 resident warps hide more of that latency
 // than 24 warps without spills do (7% faster on a dense first round).
+template <bool kFixed>
 __global__ void __launch_bounds__(kActWarps * 32, 4) k_bact(DevMatrix M, BatchState S) {
   __shared__ PairBuf s_pairs[kActWarps];
-  bact_body<false>(M, S, s_pairs);
+  bact_body<false, kFixed>(M, S, s_pairs);
 }
 
 // Three blocks per SM (80 registers): at four, 8 nodes over 2.0M nonzeros take
@@ -1105,7 +1121,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_bpersistent(DevMatrix M, BatchS
     bmark_body(M, S);
     if (!bgrid_sync(ctrl, lim)) return;
     if (split) {
-      bmark_split_body(M, S);
+      bmark_split_body<false>(M, S);
       if (!bgrid_sync(ctrl, lim)) return;
     }
     bact_body<true>(M, S, s_pairs);
@@ -1421,7 +1437,7 @@ cudaError_t launch_batch_persistent(const DevMatrix &M, const BatchState &S, int
 }
 
 cudaError_t launch_batch_round(const DevMatrix &M, const BatchState &S,
-                               cudaGraphConditionalHandle handle, int use_cond, bool few,
+                               cudaGraphConditionalHandle handle, int use_cond, ActKind kind,
                                int num_sms, cudaStream_t st, cudaEvent_t *ev) {
   cudaError_t e;
   const int64_t nslots = (int64_t)M.nslices * kSliceW;
@@ -1443,16 +1459,20 @@ cudaError_t launch_batch_round(const DevMatrix &M, const BatchState &S,
   mark(1);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   mark(2);
-  if (split)
-    k_bmark_split<<<grid_for((int64_t)M.nsplit_rows * kThreads, kThreads, num_sms * 4), kThreads,
-                    0, st>>>(M, S);
+  if (split) {
+    const int nbs = grid_for((int64_t)M.nsplit_rows * kThreads, kThreads, num_sms * 4);
+    if (kind == kActShares) k_bmark_split<true><<<nbs, kThreads, 0, st>>>(M, S);
+    else k_bmark_split<false><<<nbs, kThreads, 0, st>>>(M, S);
+  }
   mark(3);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   mark(4);
-  if (few)
+  if (kind == kActFew)
     k_bact_few<<<num_sms * 3, kActWarps * 32, 0, st>>>(M, S);
+  else if (kind == kActShares)
+    k_bact<true><<<num_sms * 4, kActWarps * 32, 0, st>>>(M, S);
   else
-    k_bact<<<num_sms * 4, kActWarps * 32, 0, st>>>(M, S);
+    k_bact<false><<<num_sms * 4, kActWarps * 32, 0, st>>>(M, S);
   mark(5);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   mark(6);

@@ -345,7 +345,7 @@ void dp_destroy(dp_ctx *ctx) {
 namespace {
 void free_batch(BatchWs *b) {
   if (!b) return;
-  for (int k = 0; k < 2; ++k) {
+  for (int k = 0; k < dp::kActKinds; ++k) {
     if (b->exec[k]) cudaGraphExecDestroy(b->exec[k]);
     if (b->graph[k]) cudaGraphDestroy(b->graph[k]);
   }
@@ -1326,19 +1326,18 @@ int ensure_batch(dp_matrix *mat, int32_t Bp) {
   return DP_OK;
 }
 
-// Makes (or reuses) the round loop of the workspace, `few` for a batch of
-// few nodes.
-int ensure_batch_graph(dp_matrix *mat, bool few) {
+// Makes (or reuses) the round loop of the workspace with the given activity kernel.
+int ensure_batch_graph(dp_matrix *mat, dp::ActKind kind) {
   BatchWs *b = mat->batch;
-  if (b->exec[few]) return DP_OK;
+  if (b->exec[kind]) return DP_OK;
   const int sms = mat->ctx->num_sms;
   const dp::DevMatrix Mc = mat->M;
   const dp::BatchState Sc = b->S;
   return build_loop_graph(
-      [Mc, Sc, sms, few](cudaGraphConditionalHandle h, cudaStream_t cs) {
-        return dp::launch_batch_round(Mc, Sc, h, 1, few, sms, cs, nullptr);
+      [Mc, Sc, sms, kind](cudaGraphConditionalHandle h, cudaStream_t cs) {
+        return dp::launch_batch_round(Mc, Sc, h, 1, kind, sms, cs, nullptr);
       },
-      &b->graph[few], &b->exec[few]);
+      &b->graph[kind], &b->exec[kind]);
 }
 
 // Device copy of a host input (staged), or the device pointer itself.
@@ -1361,7 +1360,7 @@ int stage_in(BatchWs *b, T **slot, const T *src, size_t count, size_t cap, cudaS
 
 constexpr int kBatchStages = 6;  // mark, mark_split, act, combine, cand_split, finish
 
-int batch_hostloop(dp_matrix *mat, BatchWs *b, bool few, int32_t max_rounds, float *kernel_ms,
+int batch_hostloop(dp_matrix *mat, BatchWs *b, dp::ActKind kind, int32_t max_rounds, float *kernel_ms,
                    int32_t *kernel_launches) {
   dp_ctx *ctx = mat->ctx;
   cudaStream_t st = ctx->stream;
@@ -1377,7 +1376,7 @@ int batch_hostloop(dp_matrix *mat, BatchWs *b, bool few, int32_t max_rounds, flo
   const bool launched[kBatchStages] = {true, split, true, split, split, true};
   int status = DP_OK;
   for (int32_t r = 0; r < max_rounds; ++r) {
-    cudaError_t e = dp::launch_batch_round(mat->M, b->S, 0, 0, few, ctx->num_sms, st,
+    cudaError_t e = dp::launch_batch_round(mat->M, b->S, 0, 0, kind, ctx->num_sms, st,
                                            timed ? ev : nullptr);
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(b->h_ctrl, b->S.ctrl, sizeof(dp::BCtrl), cudaMemcpyDeviceToHost, st);
@@ -1560,6 +1559,21 @@ bool teams_for_nodes(const dp_ctx *ctx, const dp_matrix *mat, int32_t count) {
 // 3866 / 2961, 20 nodes 552 / 628 and 4017 / 4472.
 constexpr int32_t kFewNodes = 16;
 
+// Work up to which a batch without long chunks has fixed shares (k_bact<true>): its
+// items times the slots of the longest.  They are even, and the ticket kernel's two
+// lists and its counter cost a round 1 to 4%; above, tickets even out the memory's
+// latencies.  Measured in us per call (tickets / shares): 90k nonzeros in rows of 5..7,
+// 256 nodes (0.84M) 2985 / 2896; 400k, 40 nodes (0.93M) 2856 / 2759, 256 nodes (3.7M)
+// 9606 / 10248; 250k in rows of 27..33, 256 nodes (2.2M) 773 / 827.
+constexpr int64_t kShareWork = 1500000;
+
+dp::ActKind act_kind(const dp::DevMatrix &M, int32_t nodes) {
+  if (nodes <= kFewNodes) return dp::kActFew;
+  const int64_t items = (int64_t)M.nslices * dp::kSliceW * ((nodes + 31) / 32);
+  return M.max_slots < dp::kTicketSlots && M.max_slots * items <= kShareWork ? dp::kActShares
+                                                                             : dp::kActTickets;
+}
+
 // How a dp_propagate_nodes call runs its rounds: the captured graph (a
 // WHILE loop of the round kernels), the host (one synchronisation per round,
 // so that each stage can be timed with CUDA events), or one persistent
@@ -1615,8 +1629,8 @@ int nodes_call(dp_ctx *ctx, const dp_matrix *cmat, int32_t count, const double *
     dp::TraceRange batch_range("node batch launch");
     const int32_t cnt = count - s0 < per ? count - s0 : per;
     const int32_t Bp = (cnt + 31) / 32 * 32;
-    const bool few = cnt <= kFewNodes;
-    if (p.max_rounds > 0 && mode == kNodesGraph && (rc = ensure_batch_graph(mat, few))) return rc;
+    const dp::ActKind kind = act_kind(mat->M, cnt);
+    if (p.max_rounds > 0 && mode == kNodesGraph && (rc = ensure_batch_graph(mat, kind))) return rc;
     const size_t off = (size_t)s0 * (size_t)n, len = (size_t)cnt * (size_t)n;
     const double *d_lb = nullptr, *d_ub = nullptr;
     if ((rc = stage_in(b, &b->st_lb, n > 0 ? lb + off : lb, len, cap, st, &d_lb))) return rc;
@@ -1642,11 +1656,11 @@ int nodes_call(dp_ctx *ctx, const dp_matrix *cmat, int32_t count, const double *
     CUDA_TRY(dp::launch_batch_prologue(mat->M, b->S, cnt, d_lb, d_ub, d_vt, d_lhs, d_rhs,
                                        p.eps_int, p.tau_rel, p.eps_feas, p.inf_threshold,
                                        ctx->num_sms, st));
-    if (p.max_rounds > 0 && mode == kNodesGraph) CUDA_TRY(cudaGraphLaunch(b->exec[few], st));
+    if (p.max_rounds > 0 && mode == kNodesGraph) CUDA_TRY(cudaGraphLaunch(b->exec[kind], st));
     if (p.max_rounds > 0 && mode == kNodesPersistent)
       CUDA_TRY(dp::launch_batch_persistent(mat->M, b->S, ctx->num_sms, st));
     if (p.max_rounds > 0 && mode == kNodesHostloop) {
-      int r2 = batch_hostloop(mat, b, few, p.max_rounds, kernel_ms, kernel_launches);
+      int r2 = batch_hostloop(mat, b, kind, p.max_rounds, kernel_ms, kernel_launches);
       if (r2) return r2;
     }
     if (n > 0) {

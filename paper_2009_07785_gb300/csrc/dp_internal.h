@@ -274,6 +274,15 @@ struct TeamArgs {
 
 // ------------------------------------------------------ batched B&B nodes --
 //
+// Which activity kernel a batched round runs; the results are the same.
+enum ActKind {
+  kActTickets,  // a chunk of one node group per warp, handed out by ticket
+  kActFew,      // batches of few nodes: chunks share warps (see k_bact_few)
+  kActShares,   // a chunk per warp in fixed shares, one list of them
+  kActKinds
+};
+constexpr int32_t kTicketSlots = 64;  // slots of a chunk from which shares are uneven
+
 // One batched call propagates Bp = 32*G bound vectors ("nodes") over one
 // matrix.  Bounds are stored node-minor, entry e = j*Bp + node, so that the
 // 32 lanes of a warp (32 nodes of one node group g) read the bounds of one

@@ -62,15 +62,13 @@ cudaError_t launch_batch_epilogue(const DevMatrix &M, const BatchState &S, int32
                                   cudaStream_t st);
 // One batched round; in a graph body (use_cond = 1) the last kernel sets
 // the WHILE condition.  With `ev` (12 events) each of the six stages (mark,
-// mark_split, act, combine, cand_split, finish) is bracketed by a pair.  With
-// `few` the chunks of a step belong to several rows (batches of few nodes,
-// see k_bact_few); the results are the same.
+// mark_split, act, combine, cand_split, finish) is bracketed by a pair.
+cudaError_t launch_batch_round(const DevMatrix &M, const BatchState &S,
+                               cudaGraphConditionalHandle handle, int use_cond, ActKind kind,
+                               int num_sms, cudaStream_t st, cudaEvent_t *ev);
 // The batch's round loop as one cooperative kernel (all rounds; no graph).
 cudaError_t launch_batch_persistent(const DevMatrix &M, const BatchState &S, int num_sms,
                                     cudaStream_t st);
-cudaError_t launch_batch_round(const DevMatrix &M, const BatchState &S,
-                               cudaGraphConditionalHandle handle, int use_cond, bool few,
-                               int num_sms, cudaStream_t st, cudaEvent_t *ev);
 
 // Serving slots (dp_batch.cu): a batch whose nodes are independent requests.
 // launch_slots_init writes the sides and types and leaves every slot empty;

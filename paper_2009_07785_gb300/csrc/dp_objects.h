@@ -74,9 +74,9 @@ struct BatchWs {
   double *st_lb = nullptr, *st_ub = nullptr, *out_lb = nullptr, *out_ub = nullptr;
   double *st_lhs = nullptr, *st_rhs = nullptr;
   uint8_t *st_vt = nullptr;
-  // round loops, [1] for batches of few nodes; each built when first needed
-  cudaGraph_t graph[2] = {nullptr, nullptr};
-  cudaGraphExec_t exec[2] = {nullptr, nullptr};
+  // round loops, by dp::ActKind; each built when first needed
+  cudaGraph_t graph[dp::kActKinds] = {};
+  cudaGraphExec_t exec[dp::kActKinds] = {};
 };
 
 namespace dp {
