@@ -56,3 +56,35 @@ def test_few_and_many_nodes_share_a_workspace(gpu):
         again = call(dp.dp_propagate_nodes, ctx, mat, inst, LB[:16], UB[:16])
     for x, y, z in zip(few, many, again):
         assert np.array_equal(x, y[:16]) and np.array_equal(x, z)
+
+
+# more work items than warps of the activity kernel (3,648), in rows of uneven length with
+# split ones among them: up to 8 nodes a step packs four chunks, up to 16 two, and
+# above the items go out in fixed shares or by ticket
+@pytest.mark.parametrize("count", [1, 7, 8, 16, 17, 40])
+@pytest.mark.parametrize("rows,chunk", [(17001, 256), (17001, 64), (9001, 16)])
+def test_batches_with_more_chunks_than_warps(gpu, orc, count, rows, chunk):
+    dp, ctx = gpu
+    rng = np.random.default_rng(rows + count)
+    lengths = np.where(rng.random(rows) < 0.02, rng.integers(40, 200, rows),
+                       rng.integers(1, 9, rows))
+    n = 12000
+    col = synth._distinct_columns(rng, lengths, n)
+    val = np.where(rng.random(col.size) < 0.5, -1.0, 1.0) * rng.integers(1, 11, col.size)
+    vt, lb, ub, x = synth._tiny_like_vars(rng, n)
+    rp = synth._row_ptr(lengths)
+    lhs, rhs = synth._sides(rng, rp, col, val, x)
+    inst = synth.Instance("few", rows, n, rp, col, val, lb, ub, vt, lhs, rhs, x)
+    LB, UB = synth.node_bounds_at_point(inst, count, seed=7)
+    with dp.Matrix(ctx, inst.m, inst.n, inst.row_ptr, inst.col, inst.val, chunk) as mat:
+        a = call(dp.dp_propagate_nodes_hostloop, ctx, mat, inst, LB, UB)
+        b = call(dp.dp_propagate_nodes_persistent, ctx, mat, inst, LB, UB)
+        c = call(dp.dp_propagate_nodes, ctx, mat, inst, LB, UB)
+    for x, y, z in zip(a, b, c):
+        assert np.array_equal(x, y) and np.array_equal(x, z)
+    for k in {0, count - 1}:
+        o = orc.propagate(inst.m, inst.n, inst.row_ptr, inst.col, inst.val, LB[k], UB[k],
+                          inst.vartype, inst.lhs, inst.rhs)
+        assert a[2][k] == o.rounds and a[3][k] == o.infeasible, k
+        nbad, _, det = compare_bounds(a[0][k], a[1][k], o.lb, o.ub, inst.vartype)
+        assert nbad == 0, det
