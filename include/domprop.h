@@ -202,7 +202,7 @@ int dp_matrix_set_compression(dp_matrix *mat, int32_t on, int32_t *active);
 typedef struct {
   int32_t chunk;        /* row split length (dp_matrix_load's `chunk`) */
   int32_t round_warps;  /* warps per block (dp_matrix_set_launch) */
-  float us_per_round;   /* measured device time of one round, microseconds */
+  float us_per_round;   /* measured time of one round, microseconds */
   int32_t reserved;
 } dp_tune_entry;
 
@@ -214,9 +214,10 @@ typedef struct {
  * Sec. 3.2: longer rows are split and combined in a second pass) and every
  * block shape {4, 8} warps, with CUDA events on each round kernel (the
  * host-driven loop; the best of three timed calls; value compression off).
- * Arguments as
- * dp_matrix_load_sides plus the problem of
- * dp_propagate; lhs/rhs order the rows when they are host arrays.
+ * A problem of few nonzeros, which dp_propagate may run on one thread block
+ * cluster (the block shape then changes nothing), is timed by whole dp_propagate
+ * calls on device-resident copies instead.  Arguments as dp_matrix_load_sides plus
+ * the problem of dp_propagate; lhs/rhs order the rows when they are host arrays.
  * entries[max_entries] (may be NULL if 0) receive the measurements, *count
  * their number, *best the fastest.  Loads and frees one matrix per
  * distinct layout, so it costs several layout builds: run it once per
@@ -239,7 +240,9 @@ int dp_autotune(dp_ctx *ctx, int32_t m, int32_t n, int64_t nnz,
  * three timed calls).  In the batched kernels a warp walks a chunk for 32
  * node lanes, so the split length bounds the serial chain of each work item:
  * short pieces suit batches with few live nodes (a server's lanes), long
- * ones batches of many nodes.  entries[].round_warps is 0 (the batched
+ * ones batches of many nodes.  (Few nodes of a small matrix, which dp_propagate_nodes
+ * runs on a cluster each, prefer pieces of 64 to 256: up to 1.4 times as fast as the
+ * shorter ones that suit the batched kernels timed here.)  entries[].round_warps is 0 (the batched
  * kernels have one launch shape); us_per_round is the batch's kernel time
  * divided by its rounds.  Other arguments and results as dp_autotune.
  */

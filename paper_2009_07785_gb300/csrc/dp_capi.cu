@@ -995,8 +995,8 @@ int dp_propagate(dp_ctx *ctx, const dp_matrix *cmat, const double *lb,
                       infeasible, rounds, &p);
   if (rc) return rc;
   dp_matrix *mat = const_cast<dp_matrix *>(cmat);
-  if (mat->h_res && mat->ninst == 0 && !mat->M.val8 && mat->M.nnz <= kTeamNnz &&
-      mat->M.nslices <= kTeamSlices && ctx->teams_of[0] > 0) {
+  if (mat->h_res && mat->ninst == 0 && !mat->M.val8 && mat->M.nslices <= kTeamSlices &&
+      dp::single_may_be_team(ctx, mat->M.nnz)) {
     rc = team_call(ctx, mat, lb, ub, vartype, lhs, rhs, p, lb_out, ub_out);
     if (rc) return rc;
     *infeasible = mat->h_res->x;
@@ -1182,6 +1182,10 @@ int dp_propagate_hostloop(dp_ctx *ctx, const dp_matrix *cmat, const double *lb,
 // ------------------------------------------------------ batched B&B nodes --
 
 namespace dp {
+
+bool single_may_be_team(const dp_ctx *ctx, int64_t nnz) {
+  return nnz <= kTeamNnz && ctx->teams_of[0] > 0;
+}
 
 bool is_device_ptr(const void *p) {
   cudaPointerAttributes a;

@@ -90,5 +90,7 @@ int alloc_batch_state(const DevMatrix &M, int32_t Bp, std::vector<void *> &alloc
 size_t batch_state_bytes(const DevMatrix &M, int32_t Bp);
 // True for device (or managed) memory.
 bool is_device_ptr(const void *p);
+// Whether dp_propagate may run a problem of nnz nonzeros as one team.
+bool single_may_be_team(const dp_ctx *ctx, int64_t nnz);
 
 }  // namespace dp

@@ -143,3 +143,27 @@ def test_cluster_is_sized_by_long_chunks(gpu):
             call.append((time.perf_counter() - t0) * 1e3)
             loop.append(sum(dp.dp_propagate_hostloop(ctx, mat, *d, timing=True).kernel_ms))
     assert min(call) < 1.6 * min(loop), (min(call), min(loop))
+
+
+def test_autotune_times_the_path_that_runs(gpu):
+    """A problem that dp_propagate gives to a cluster is tuned by its calls: every
+    entry's time is that of a call with its layout (the host-driven loop's kernels
+    take up to twice as long on it)."""
+    dp, ctx = gpu
+    inst = synth.large(scale=0.00125)
+    assert inst.nnz <= 100_000
+    t = dp.dp_autotune(ctx, inst.m, inst.n, inst.row_ptr, inst.col, inst.val, inst.lb, inst.ub,
+                       inst.vartype, inst.lhs, inst.rhs)
+    assert {e["round_warps"] for e in t["entries"]} == {4, 8}
+    assert len({e["chunk"] for e in t["entries"]}) >= 3
+    d = [dev(a) for a in inst.problem()]
+    for e in t["entries"]:
+        with dp.Matrix(ctx, inst.m, inst.n, inst.row_ptr, inst.col, inst.val, e["chunk"], inst.lhs,
+                       inst.rhs) as mat:
+            best = []
+            for _ in range(8):
+                t0 = time.perf_counter()
+                r = dp.dp_propagate(ctx, mat, *d)
+                best.append((time.perf_counter() - t0) * 1e6)
+        ratio = e["us_per_round"] * r.rounds / min(best)
+        assert 0.6 < ratio < 1.4, (e, min(best), r.rounds)
