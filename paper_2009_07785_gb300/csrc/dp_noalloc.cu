@@ -210,8 +210,8 @@ constexpr int kNaUnroll = 4;     // nonzeros whose loads are in flight together
 constexpr int kNaLaneRow = 32;   // longest row that one lane takes
 constexpr int kNaWarpRow = 256;  // longest row that one warp takes
 // What a row costs, in 0.062 us: a lane 2.1 us per nonzero (its candidates'
-// divisions, whatever the other lanes do), a warp 4 us and 0.062 us per nonzero, a
-// block 8 us and 0.012 us per nonzero.
+// divisions, whatever the other lanes do), a warp 4 us and 0.06 (few accepted
+// candidates) to 0.12 us per nonzero, a block 8 us and 0.012 us per nonzero.
 constexpr unsigned kNaLaneCost = 34, kNaWarpCost = 64, kNaBlockCost = 130, kNaBlockShare = 5;
 
 // Loads nonzeros k, k + step, ... (kNaUnroll of them, those below e).
@@ -373,12 +373,6 @@ k_na_round(int32_t m, int per, const int64_t *row_ptr, const double *lhs_in,
   __shared__ int s_count;
   __shared__ unsigned s_rest;
   __shared__ unsigned long long s_cost, s_top;
-  if (threadIdx.x == 0) {
-    s_count = 0;
-    s_rest = 0u;
-    s_cost = s_top = 0ull;
-  }
-  __syncthreads();
   const int64_t i = blockIdx.x * (int64_t)per + threadIdx.x;
   NaRow r;
   r.minfin = r.maxfin = r.lhs = r.rhs = 0.0;
@@ -392,25 +386,34 @@ k_na_round(int32_t m, int per, const int64_t *row_ptr, const double *lhs_in,
     e = row_ptr[i + 1];
   }
   const unsigned long long len = (unsigned long long)(e - b);
-  if (len > kNaWarpRow) {
-    s_long[atomicAdd(&s_count, 1)] = threadIdx.x;
-    atomicAdd(&s_cost, kNaBlockCost + len / kNaBlockShare);
-    atomicMax(&s_top, len);
+  const bool is_long = len > kNaWarpRow;
+  bool by_block = false;  // the block takes its long rows one after the other
+  if (__syncthreads_or(is_long)) {
+    if (threadIdx.x == 0) {
+      s_count = 0;
+      s_rest = 0u;
+      s_cost = s_top = 0ull;
+    }
+    __syncthreads();
+    if (is_long) {
+      s_long[atomicAdd(&s_count, 1)] = threadIdx.x;
+      atomicAdd(&s_cost, kNaBlockCost + len / kNaBlockShare);
+      atomicMax(&s_top, len);
+    }
+    const unsigned most = __reduce_max_sync(full, is_long ? 0u : (unsigned)len);
+    if ((threadIdx.x & 31) == 0) atomicMax(&s_rest, most);
+    __syncthreads();
+    // else they lengthen the lanes' walk
+    by_block = s_cost < kNaLaneCost * (s_top - s_rest);
   }
-  const unsigned most = __reduce_max_sync(full, len > kNaWarpRow ? 0u : (unsigned)len);
-  if ((threadIdx.x & 31) == 0) atomicMax(&s_rest, most);
-  __syncthreads();
-  // whether the block takes its long rows one after the other, or a lane each,
-  // which lengthens the lanes' walk
-  const bool by_block = s_cost < kNaLaneCost * (s_top - s_rest);
   // the rows left to this warp: the mid ones by the warp one after the other, or
   // by a lane each like the others
-  const unsigned wlen = len > kNaWarpRow && by_block ? 0u : (unsigned)min(len, 1ull << 26);
-  const bool mid = len > kNaLaneRow && len <= kNaWarpRow;
+  const unsigned wlen = is_long && by_block ? 0u : (unsigned)min(len, 1ull << 26);
+  const bool mid = len > kNaLaneRow && !is_long;
   const unsigned rest = __reduce_max_sync(full, mid ? 0u : wlen);
-  const bool by_warp = kNaLaneCost * rest + __reduce_add_sync(full, mid ? kNaWarpCost + wlen : 0u) <
+  const bool by_warp = kNaLaneCost * rest + __reduce_add_sync(full, mid ? kNaWarpCost + 2u * wlen : 0u) <
                        kNaLaneCost * __reduce_max_sync(full, wlen);
-  if (have && !(mid && by_warp) && !(len > kNaWarpRow && by_block)) na_row_lane(A, r, b, e);
+  if (have && !(mid && by_warp) && !(is_long && by_block)) na_row_lane(A, r, b, e);
   __syncwarp();
   unsigned todo = __ballot_sync(full, mid && by_warp);
   for (; todo != 0u; todo &= todo - 1u) {
