@@ -1109,7 +1109,8 @@ __device__ __forceinline__ bool bgrid_sync(BCtrl *c, long long limit) {
 // kernel for all rounds).  Each phase is the body of the graph kernel of
 // the same name, grid-strided over the resident blocks, with a grid barrier
 // between phases instead of a kernel boundary; block 0 ends each round.
-// Four blocks per SM, as k_bact.
+// Four blocks per SM, as k_bact.  kFixed: fixed shares of the work items.
+template <bool kFixed>
 __global__ void __launch_bounds__(kThreads, 4) k_bpersistent(DevMatrix M, BatchState S) {
   __shared__ PairBuf s_pairs[kThreads / 32];
   __shared__ uint32_t s_chg[kMaxGroups], s_inf[kMaxGroups];
@@ -1121,10 +1122,10 @@ __global__ void __launch_bounds__(kThreads, 4) k_bpersistent(DevMatrix M, BatchS
     bmark_body(M, S);
     if (!bgrid_sync(ctrl, lim)) return;
     if (split) {
-      bmark_split_body<false>(M, S);
+      bmark_split_body<kFixed>(M, S);
       if (!bgrid_sync(ctrl, lim)) return;
     }
-    bact_body<true>(M, S, s_pairs);
+    bact_body<true, kFixed>(M, S, s_pairs);
     if (!bgrid_sync(ctrl, lim)) return;
     if (split) {
       bcombine_body(M, S);
@@ -1422,18 +1423,26 @@ cudaError_t launch_batch_epilogue(const DevMatrix &M, const BatchState &S, int32
   return cudaGetLastError();
 }
 
-cudaError_t launch_batch_persistent(const DevMatrix &M, const BatchState &S, int num_sms,
-                                    cudaStream_t st) {
+// Work items up to which the persistent loop deals them out in fixed shares.  Measured
+// in us per call (tickets / shares), irregular systems: 195k nonzeros, 8 nodes 4624 /
+// 4190, 256 nodes (160,000 items) 8941 / 8666; 2.0M, 64 nodes (400,000) 13818 / 14191,
+// 256 nodes 44003 / 47200.
+constexpr int64_t kPersistentShareItems = 250000;
+
+cudaError_t launch_batch_persistent(const DevMatrix &M, const BatchState &S, int32_t nodes,
+                                    int num_sms, cudaStream_t st) {
+  const bool fixed =
+      (int64_t)M.nslices * kSliceW * ((nodes + 31) / 32) <= kPersistentShareItems;
+  const void *kern =
+      fixed ? (const void *)k_bpersistent<true> : (const void *)k_bpersistent<false>;
   int per_sm = 0;
-  cudaError_t e =
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bpersistent, kThreads, 0);
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, 0);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorLaunchOutOfResources;
   DevMatrix m = M;
   BatchState s = S;
   void *args[] = {&m, &s};
-  return cudaLaunchCooperativeKernel((const void *)k_bpersistent, dim3(num_sms * per_sm),
-                                     dim3(kThreads), args, 0, st);
+  return cudaLaunchCooperativeKernel(kern, dim3(num_sms * per_sm), dim3(kThreads), args, 0, st);
 }
 
 cudaError_t launch_batch_round(const DevMatrix &M, const BatchState &S,

@@ -1662,7 +1662,7 @@ int nodes_call(dp_ctx *ctx, const dp_matrix *cmat, int32_t count, const double *
                                        ctx->num_sms, st));
     if (p.max_rounds > 0 && mode == kNodesGraph) CUDA_TRY(cudaGraphLaunch(b->exec[kind], st));
     if (p.max_rounds > 0 && mode == kNodesPersistent)
-      CUDA_TRY(dp::launch_batch_persistent(mat->M, b->S, ctx->num_sms, st));
+      CUDA_TRY(dp::launch_batch_persistent(mat->M, b->S, cnt, ctx->num_sms, st));
     if (p.max_rounds > 0 && mode == kNodesHostloop) {
       int r2 = batch_hostloop(mat, b, kind, p.max_rounds, kernel_ms, kernel_launches);
       if (r2) return r2;

@@ -67,8 +67,8 @@ cudaError_t launch_batch_round(const DevMatrix &M, const BatchState &S,
                                cudaGraphConditionalHandle handle, int use_cond, ActKind kind,
                                int num_sms, cudaStream_t st, cudaEvent_t *ev);
 // The batch's round loop as one cooperative kernel (all rounds; no graph).
-cudaError_t launch_batch_persistent(const DevMatrix &M, const BatchState &S, int num_sms,
-                                    cudaStream_t st);
+cudaError_t launch_batch_persistent(const DevMatrix &M, const BatchState &S, int32_t nodes,
+                                    int num_sms, cudaStream_t st);
 
 // Serving slots (dp_batch.cu): a batch whose nodes are independent requests.
 // launch_slots_init writes the sides and types and leaves every slot empty;

@@ -58,14 +58,8 @@ def test_few_and_many_nodes_share_a_workspace(gpu):
         assert np.array_equal(x, y[:16]) and np.array_equal(x, z)
 
 
-# more work items than warps of the activity kernel (3,648), in rows of uneven length with
-# split ones among them: up to 8 nodes a step packs four chunks, up to 16 two, and
-# above the items go out in fixed shares or by ticket
-@pytest.mark.parametrize("count", [1, 7, 8, 16, 17, 40])
-@pytest.mark.parametrize("rows,chunk", [(17001, 256), (17001, 64), (9001, 16)])
-def test_batches_with_more_chunks_than_warps(gpu, orc, count, rows, chunk):
-    dp, ctx = gpu
-    rng = np.random.default_rng(rows + count)
+def uneven(rows, seed):
+    rng = np.random.default_rng(seed)
     lengths = np.where(rng.random(rows) < 0.02, rng.integers(40, 200, rows),
                        rng.integers(1, 9, rows))
     n = 12000
@@ -74,7 +68,19 @@ def test_batches_with_more_chunks_than_warps(gpu, orc, count, rows, chunk):
     vt, lb, ub, x = synth._tiny_like_vars(rng, n)
     rp = synth._row_ptr(lengths)
     lhs, rhs = synth._sides(rng, rp, col, val, x)
-    inst = synth.Instance("few", rows, n, rp, col, val, lb, ub, vt, lhs, rhs, x)
+    return synth.Instance("few", rows, n, rp, col, val, lb, ub, vt, lhs, rhs, x)
+
+
+# more work items than warps of the activity kernel (3,648), in rows of uneven length with
+# split ones among them: up to 8 nodes a step packs four chunks, up to 16 two, and
+# above the items go out in fixed shares or by ticket (the persistent loop's from
+# 250,000 items on)
+@pytest.mark.parametrize("rows,chunk,count",
+                         [(r, c, k) for r, c in ((17001, 256), (17001, 64), (9001, 16))
+                          for k in (1, 7, 8, 16, 17, 40)] + [(17001, 64, 480)])
+def test_batches_with_more_chunks_than_warps(gpu, orc, count, rows, chunk):
+    dp, ctx = gpu
+    inst = uneven(rows, seed=rows + count)
     LB, UB = synth.node_bounds_at_point(inst, count, seed=7)
     with dp.Matrix(ctx, inst.m, inst.n, inst.row_ptr, inst.col, inst.val, chunk) as mat:
         a = call(dp.dp_propagate_nodes_hostloop, ctx, mat, inst, LB, UB)
