@@ -494,11 +494,6 @@ __device__ __forceinline__ void acc_nnz(double av, double L, double U, float WU,
 template <bool kVal8>
 using Raw = typename std::conditional<kVal8, int, double>::type;
 template <bool kVal8>
-__device__ __forceinline__ Raw<kVal8> ld_raw(const DevMatrix &M, int64_t off) {
-  if constexpr (kVal8) return (int)__ldcs(M.val8 + off);
-  else return __ldcs(M.val + off);
-}
-template <bool kVal8>
 __device__ __forceinline__ double coef_of(Raw<kVal8> r) {
   if constexpr (kVal8) return small_int_to_double(r);
   else return r;
@@ -553,16 +548,12 @@ __device__ __forceinline__ RowView whole_row(const ChunkHead &h, const ChunkAcc 
 constexpr int kTeamU = 2;            // slots per warp and step
 constexpr int kTeamBlocksPerSM = 4;  // long slices per SM up to which a block takes each
 
-struct TeamPart {  // one warp's share of a chunk
-  ChunkAcc r;
-};
-
 template <int kWarps>
 struct TeamBuf {
   static constexpr int kStep = kWarps * kTeamU;
   union {
     double b[2][2][kStep][kSliceW];      // [side][buffer][slot][lane] bounds of a step
-    TeamPart part[kWarps][kSliceW];
+    ChunkAcc part[kWarps][kSliceW];      // the warps' shares of the chunks
   };
   double fin[2][kSliceW];
   RowView rv[kSliceW];
@@ -658,14 +649,14 @@ __device__ __forceinline__ void team_slice(const DevMatrix &M, const DevState &S
     if (need_max && warp == wmax) chain(last, 1);
     __syncthreads();  // the staging is free for the warps' parts
   }
-  sb.part[warp][lane].r = r;
+  sb.part[warp][lane] = r;
   if (warp == wmin) sb.fin[0][lane] = need_min ? fin : 0.0;
   if (kWarps > 1 && warp == wmax) sb.fin[1][lane] = need_max ? fin : 0.0;
   __syncthreads();
   if (warp == 0) {
 #pragma unroll 1
     for (int w = 1; w < kWarps; ++w) {
-      const ChunkAcc q = sb.part[w][lane].r;
+      const ChunkAcc q = sb.part[w][lane];
       if (q.mininf > 0) r.t.kinf_min = q.t.kinf_min;
       if (q.maxinf > 0) r.t.kinf_max = q.t.kinf_max;
       r.mininf += q.mininf;
@@ -701,7 +692,6 @@ __device__ __forceinline__ void team_slice(const DevMatrix &M, const DevState &S
 // shuffled values (lanes below 16 add up the minimum activity, the others
 // the maximum): the same FMA chain in CSR order, 64 clocks per slot, where a
 // lane alone takes about 310 (256 slots: 12-20 us instead of 75).
-template <bool kVal8, bool kCo>
 __device__ __forceinline__ void coop_activity(const DevMatrix &M, const VarRec *rec,
                                               int64_t elem0, int32_t len, bool need_min,
                                               bool need_max, ChunkAcc &r, double &minfin,
@@ -729,7 +719,7 @@ __device__ __forceinline__ void coop_activity(const DevMatrix &M, const VarRec *
     uint32_t fl;
 #pragma unroll
     for (int u = 0; u < 4; ++u)
-      if (t0 + 32 * u + lane < len) ld_rec_t<kCo>(rec + j[u], L[u], U[u], WU[u], WL[u], fl);
+      if (t0 + 32 * u + lane < len) ld_rec(rec + j[u], L[u], U[u], WU[u], WL[u], fl);
 #pragma unroll
     for (int u = 0; u < 4; ++u)
       if (t0 + 32 * u + lane < len)
@@ -765,7 +755,7 @@ __device__ __forceinline__ void coop_activity(const DevMatrix &M, const VarRec *
 }
 
 // A marked chunk of a long slice (warp-level).
-template <bool kMulti, bool kVal8>
+template <bool kMulti>
 __device__ __forceinline__ void coop_chunk(const DevMatrix &M, const DevState &S, int slice,
                                            int which) {
   const int lane = threadIdx.x & 31;
@@ -787,7 +777,7 @@ __device__ __forceinline__ void coop_chunk(const DevMatrix &M, const DevState &S
   const int64_t elem0 = M.slice_off[slice] + which;
   ChunkAcc r;
   double minfin, maxfin;
-  coop_activity<kVal8, false>(M, S.rec, elem0, h.len, d_isfinite(h.sd.y), d_isfinite(h.sd.x), r,
+  coop_activity(M, S.rec, elem0, h.len, d_isfinite(h.sd.y), d_isfinite(h.sd.x), r,
                               minfin, maxfin);
   if (h.exact) r.t.r1 = r.t.r2 = r.t.l1 = r.t.l2 = f_inf();
   if (slice < M.nslices_split) {
@@ -865,7 +855,7 @@ k_round(DevMatrix M, DevState S, int few) {
     uint32_t m = s_bits;
     if (__popc(m) <= kRoundWarps) {  // few chunks: one per warp
       for (int at = 0; m != 0u; m &= m - 1u, ++at)
-        if (at == warp) coop_chunk<kMulti, kVal8>(M, S, slice, __ffs(m) - 1);
+        if (at == warp) coop_chunk<kMulti>(M, S, slice, __ffs(m) - 1);
     } else {
       team_slice<kMulti, kRoundWarps, kVal8>(M, S, slice, m, sb);
     }

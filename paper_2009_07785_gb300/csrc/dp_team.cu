@@ -194,15 +194,14 @@ __device__ __forceinline__ bool push_named(const TeamArgs &A, const Team &T, Pai
   return full;
 }
 
-// Re-reads the lanes' chunks (len slots each, 0 for none) and buffers every
-// nonzero that survives: kU slots from kbeg, then every kstep further on.
-// All 32 lanes call.
+// Re-reads the lanes' chunks (len slots each, 0 for none), kU slots at a time, and
+// buffers every nonzero that survives.  All 32 lanes call.
 __device__ __forceinline__ void push_reread(const TeamArgs &A, const Team &T, Pairs &B, int &n,
-                                            const RowView &rv, int32_t len, int kbeg, int kstep,
-                                            int64_t slot, int64_t elem0) {
+                                            const RowView &rv, int32_t len, int64_t slot,
+                                            int64_t elem0) {
   constexpr int kU = 4;
   const int maxlen = __reduce_max_sync(kFull, len);
-  for (int k = kbeg; k < maxlen; k += kstep) {
+  for (int k = 0; k < maxlen; k += kU) {
     double a[kU], L[kU], U[kU];
     float WU[kU], WL[kU];
     int32_t j[kU];
@@ -434,7 +433,7 @@ __device__ __noinline__ int slice_by_lanes(const TeamArgs &A, const Team &T, Pai
   const RowView rv = whole_row(A, T, h, r, minfin, maxfin, true);
   const bool full = push_named(A, T, B, n, rv, r.t, r.mininf, r.maxinf, h.c, h.elem0);
   if (__ballot_sync(kFull, full) != 0u)
-    push_reread(A, T, B, n, rv, full ? len : 0, 0, 4, h.c, h.elem0);
+    push_reread(A, T, B, n, rv, full ? len : 0, h.c, h.elem0);
   return n;
 }
 
@@ -790,7 +789,7 @@ __device__ __noinline__ int split_candidates(const TeamArgs &A, const Team &T, P
     const int64_t elem0 = __ldg(A.M.slice_off + slice) + lane;
     const bool full = push_named(A, T, B, n, rv, t, cmin, cmax, c, elem0);
     if (__ballot_sync(kFull, full) == 0u) continue;
-    push_reread(A, T, B, n, rv, full ? len : 0, 0, 4, c, elem0);
+    push_reread(A, T, B, n, rv, full ? len : 0, c, elem0);
   }
   return n;
 }
