@@ -460,8 +460,8 @@ void worker_main(dp_server *s) {
 bool finite_request(const double *lb, const double *ub, int32_t n, double thr) {
   // the caller's thread pays for this on every request: without an exit per
   // entry the comparisons vectorise (a NaN fails either).  A burst of 256
-  // requests of 7k variables on average: 3.4 -> 2.4 ms of submission, 8.2 -> 7.3
-  // ms until all are answered.
+  // requests of 7k variables on average: 3.4 -> 2.4 ms of submission (of 8.6 until
+  // all are answered, which did not change beyond the runs' spread).
   constexpr int32_t kBlock = 512;
   for (int32_t j0 = 0; j0 < n; j0 += kBlock) {
     const int32_t j1 = std::min(n, j0 + kBlock);
