@@ -106,7 +106,8 @@ constexpr int32_t kMarkShare = 32;
 //                 nodes 3235 / 1269 and 171 / 204; 250k, 1 node 2928 / 1573 and 175 /
 //                 226, 16 nodes 3267 / 2933;
 //                 short rows 60k, 8 nodes 734 / 472, 33 nodes 953 / 672, 100 nodes
-//                 1369 / 1622; 140k, 8 nodes 823 / 725, 16 nodes 908 / 1094;
+//                 1369 / 1622; 90k, 12 nodes 780 / 611 (3.7 slices per warp), 16
+//                 nodes 764 / 811 (7.3);
 //                 1000 nodes over 2k in rows of 6 1545 / 927 (10 items), of 30 387 /
 //                 712 (34 items); over 4k in rows of 4 2372 / 1824 (31 items), over 12k in
 //                 rows of 6 2274 / 2837 (63 items)
@@ -126,6 +127,7 @@ constexpr int64_t kTeamNodeNnz = 300000;   // the matrix of a node batch with lo
 constexpr int64_t kTeamNodeWork = 2500000;  // nonzeros times nodes: up to kTeamNnz nonzeros,
 constexpr int64_t kTeamNodeWorkLong = 1000000;  // and above
 constexpr int64_t kTeamNodeItems = 32;     // team_items of a matrix with more nodes than teams
+constexpr int64_t kTeamNodeShare = 6;      // team_items per warp without long slices
 constexpr int kTeamWarps = 8;  // warps per block of a team
 
 // What the warps of a team share out in a round: the slices, the long ones
@@ -1548,11 +1550,14 @@ int nodes_by_teams(dp_ctx *ctx, dp_matrix *mat, int32_t count, const double *lb,
 bool teams_for_nodes(const dp_ctx *ctx, const dp_matrix *mat, int32_t count) {
   if (!mat->h_res || ctx->teams_of[0] <= 0) return false;
   const int64_t nnz = mat->M.nnz, work = nnz * (int64_t)count;
+  const int64_t items = team_items(mat->M.nslices, mat->M.nlong);
   // teams of one block take the nodes in several turns
-  if (count > ctx->teams_of[0] && team_items(mat->M.nslices, mat->M.nlong) > kTeamNodeItems)
-    return false;
-  if (nnz <= kTeamNnz) return work <= kTeamNodeWork;
-  return mat->M.nlong > 0 && nnz <= kTeamNodeNnz && work <= kTeamNodeWorkLong;
+  if (count > ctx->teams_of[0] && items > kTeamNodeItems) return false;
+  if (mat->M.nlong == 0)
+    return nnz <= kTeamNnz && work <= kTeamNodeWork &&
+           items <= (int64_t)kTeamNodeShare * (kTeamWarps << team_size(ctx, items, count));
+  return nnz <= kTeamNnz ? work <= kTeamNodeWork
+                         : nnz <= kTeamNodeNnz && work <= kTeamNodeWorkLong;
 }
 
 // Nodes up to which a batch's chunks share warps (k_bact_few).  Measured in us
